@@ -54,7 +54,7 @@ def listed():
          "block": 24, "maxit": 6},
         # A share of the sweep: problems with their own windows, strengths and phases in one
         # mixed-precision call, to convergence; eigenvalues are what the sweep keeps.
-        {"name": "sweep_mixed", "kind": "sweep", "KLs": "5,6,7,8", "nev": 16, "block": 24},
+        {"name": "sweep_mixed", "kind": "sweep", "KLs": "5,6,7,6", "nev": 16, "block": 24},
         # One step of the warm-start network: loss and all gradients of a batch.
         {"name": "warmstart_step", "kind": "step", "hidden": 512, "layers": 4, "nvec": 16,
          "ncore": 256, "batch": 256},
@@ -116,7 +116,7 @@ def draw(rng):
                 "eps": round(rng.uniform(0.3, 6.0), 3), "nev": nev,
                 "block": min(24, nev + rng.randint(2, 8)), "maxit": rng.randint(5, 7)}
     if kind == "sweep":
-        n = rng.randint(2, 4)
+        n = rng.randint(2, 3)
         return {"kind": "sweep", "KLs": ",".join(str(rng.choice([5, 5, 6])) for _ in range(n)),
                 "nev": 16, "block": 24}
     return {"kind": "step", "hidden": 64 * rng.randint(2, 8), "layers": rng.randint(2, 4),
