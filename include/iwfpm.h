@@ -191,7 +191,7 @@ typedef struct {
  * for iwf_preconditioner. Every step runs on the device: the FFT apply, the residual and
  * preconditioner, Gram products and block updates (IWF_PREC_F64: tensor cores, FP64 values
  * split into 56-bit fixed-point bf16 digits, Ozaki scheme), orthonormalisation and the small
- * Rayleigh-Ritz eigenproblem (one-CTA Jacobi, FP64 angles, double-float rotations); the host
+ * Rayleigh-Ritz eigenproblem (one CTA, FP64: Householder, bisection, inverse iteration); the host
  * reads only the residual norms once per iteration.
  *   X0     device, N*block complex doubles (window order, column-major) or NULL for a seeded
  *          random start (splitmix64 counter generator).

@@ -23,50 +23,11 @@ template <> struct Acc<float> { using type = float; };
 // this form (about 48 FP32 operations) costs about a fifth of its 4 FP64 fmas.
 struct DF4 { float rh, rl, ih, il; };              // complex: re (hi, lo), im (hi, lo)
 
-// x = hi + lo with integer and FP32 operations only: conversions between double and float,
-// and double arithmetic, issue on the slow FP64 pipe and made the staging of a tile cost as
-// much as its products. hi is x truncated to 24 significant bits (built from x's sign,
-// exponent and top fraction bits); lo is the remaining 29 fraction bits rounded to a float
-// (two exact 23-bit integer-to-float conversions by the 2^23 bias trick and one fma) times
-// the exact power of two 2^(e - 52). |x| < 2^-126 gives (0, 0); below 2^-75 lo is 0.
-__device__ __forceinline__ void split_bits(double x, float& hi, float& lo) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const unsigned int hw = (unsigned int)(b >> 32), lw = (unsigned int)b;
-  const int e = (int)((hw >> 20) & 0x7ffu);          // biased exponent
-  const unsigned int sign = hw & 0x80000000u;
-  if (e < 1023 - 126) { hi = 0.f; lo = 0.f; return; }
-  const unsigned int top23 = ((hw & 0xfffffu) << 3) | (lw >> 29);
-  hi = __uint_as_float(sign | ((unsigned int)(e - 1023 + 127) << 23) | top23);
-  const unsigned int rest = lw & 0x1fffffffu;
-  const float rh = __uint_as_float(0x4B000000u | (rest >> 23)) - 8388608.f;      // exact
-  const float rl = __uint_as_float(0x4B000000u | (rest & 0x7fffffu)) - 8388608.f;  // exact
-  const float r = fmaf(rh, 8388608.f, rl);
-  const int se = e - 1075 + 127;
-  const float scale = se > 0 ? __uint_as_float((unsigned int)se << 23) : 0.f;
-  lo = r * scale;
-  if (sign) lo = -lo;
-}
 __device__ __forceinline__ DF4 df_split(double2 v) {
   DF4 o;
   split_bits(v.x, o.rh, o.rl);
   split_bits(v.y, o.ih, o.il);
   return o;
-}
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = a + b;
-  const float bb = s - a;
-  e = (a - (s - bb)) + (b - bb);
-}
-// (sh, sl) += (xh + xl)(yh + yl), dropping xl*yl (below 2^-48 relative)
-__device__ __forceinline__ void df_mac(float& sh, float& sl, float xh, float xl, float yh, float yl) {
-  const float p = xh * yh;
-  float t = fmaf(xh, yh, -p);                      // exact: xh*yh = p + t
-  t = fmaf(xh, yl, t);
-  t = fmaf(xl, yh, t);
-  float s, e;
-  two_sum(sh, p, s, e);
-  sh = s;
-  sl += e + t;
 }
 __device__ __forceinline__ double df_value(float h, float l) { return (double)h + (double)l; }
 
@@ -456,441 +417,6 @@ __global__ void resid_finish(Batch bt, const double* partial, int slots, int b, 
   resid[(size_t)prob * kMaxBlock + j] = sqrt(s);
 }
 
-// ---------------------------------------------------------------------------------------
-// One-CTA dense Hermitian eigensolver: parallel cyclic Jacobi (round-robin pairing), FP64.
-// A (n x n, row-major, leading dimension ld) is overwritten; V receives the eigenvectors.
-constexpr int kSmallThreads = 512;
-
-struct SmallShared {
-  double2 A[kMaxSmall * kMaxSmall];
-  double2 V[kMaxSmall * kMaxSmall];
-  double2 B[kMaxSmall * kMaxBlock];   // m x b scratch (the P coefficients)
-  double w[kMaxSmall];
-  double w2[kMaxSmall];
-  double d[kMaxSmall];
-  float4 rot_cs[kMaxSmall / 2 + 1];   // Jacobi: c and s as float pairs (c.h, c.l, s.h, s.l)
-  float4 rot_ph[kMaxSmall / 2 + 1];   // Jacobi: e^{-i phi} as float pairs (re.h, re.l, im.h, im.l)
-  int rp[kMaxSmall / 2 + 1], rq[kMaxSmall / 2 + 1];
-  int idx[kMaxSmall];
-  int perm[kMaxSmall];
-  double red[kSmallThreads / 32];
-  int flag;
-  int rot;
-};
-
-__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
-  return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-__device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
-
-__device__ double block_sum(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = v;
-  __syncthreads();
-  double s = 0;
-  for (int w = 0; w < (int)(blockDim.x / 32); ++w) s += red[w];
-  __syncthreads();
-  return s;
-}
-
-// ---- double-float scalars for the Jacobi rotations ---------------------------------------
-struct DF { float h, l; };
-__device__ __forceinline__ DF df_of(double x) {
-  DF o;
-  o.h = __double2float_rn(x);
-  o.l = __double2float_rn(x - (double)o.h);
-  return o;
-}
-__device__ __forceinline__ double df_dbl(DF a) { return (double)a.h + (double)a.l; }
-__device__ __forceinline__ DF df_norm(float s, float e) {   // fast two-sum, |s| >= |e|
-  DF o;
-  o.h = s + e;
-  o.l = e - (o.h - s);
-  return o;
-}
-__device__ __forceinline__ DF df_mul(DF a, DF b) {
-  const float p = a.h * b.h;
-  float e = fmaf(a.h, b.h, -p);
-  e = fmaf(a.h, b.l, e);
-  e = fmaf(a.l, b.h, e);
-  return df_norm(p, e);
-}
-__device__ __forceinline__ DF df_add(DF a, DF b) {
-  float s, e;
-  two_sum(a.h, b.h, s, e);
-  e += a.l + b.l;
-  return df_norm(s, e);
-}
-__device__ __forceinline__ DF df_neg(DF a) { return DF{-a.h, -a.l}; }
-// complex double-float, stored in the 16 bytes of a double2
-struct CDF { DF re, im; };
-__device__ __forceinline__ CDF cdf_mul(CDF a, CDF b) {
-  return CDF{df_add(df_mul(a.re, b.re), df_neg(df_mul(a.im, b.im))),
-             df_add(df_mul(a.re, b.im), df_mul(a.im, b.re))};
-}
-// c a - s t and s a + c t for real c, s
-__device__ __forceinline__ void cdf_rot(CDF a, CDF t, DF c, DF s, CDF& a2, CDF& t2) {
-  a2 = CDF{df_add(df_mul(c, a.re), df_neg(df_mul(s, t.re))),
-           df_add(df_mul(c, a.im), df_neg(df_mul(s, t.im)))};
-  t2 = CDF{df_add(df_mul(s, a.re), df_mul(c, t.re)), df_add(df_mul(s, a.im), df_mul(c, t.im))};
-}
-__device__ __forceinline__ CDF& cdf_at(double2* base, int e) {
-  return *reinterpret_cast<CDF*>(base + e);
-}
-__device__ __forceinline__ CDF cdf_of(double2 v) { return CDF{df_of(v.x), df_of(v.y)}; }
-__device__ __forceinline__ double2 dbl_of(CDF v) { return make_double2(df_dbl(v.re), df_dbl(v.im)); }
-
-// Eigen-decomposition of the Hermitian n x n matrix in sh.A (row-major, ld = n).
-// On return sh.w holds ascending eigenvalues and sh.V (row-major) the eigenvectors as columns.
-// The rotations run in double-float arithmetic on the FP32 pipes (A and V are held as float
-// pairs in place of their double2 entries while the sweeps run): this one-CTA solve sits on
-// the critical path of every iteration, and FP64 on this GPU issues at 1/62 of the FP32 rate.
-// Rotation angles are computed in FP64 from the double-float entries.
-__device__ void jacobi_eig(SmallShared& sh, int n) {
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int e = tid; e < n * n; e += nt) {
-    const int i = e / n, j = e % n;
-    sh.V[e] = make_double2(i == j ? 1.0 : 0.0, 0.0);
-    // symmetrise: A = (A + A^H)/2
-    if (i < j) {
-      const double2 a = sh.A[i * n + j], c = sh.A[j * n + i];
-      const double2 m = make_double2(0.5 * (a.x + c.x), 0.5 * (a.y - c.y));
-      sh.A[i * n + j] = m;
-      sh.A[j * n + i] = cconj(m);
-    } else if (i == j) {
-      sh.A[e].y = 0.0;
-    }
-  }
-  __syncthreads();
-  if (n == 1) {
-    if (tid == 0) sh.w[0] = sh.A[0].x;
-    __syncthreads();
-    return;
-  }
-  for (int e = tid; e < n * n; e += nt) {
-    cdf_at(sh.A, e) = cdf_of(sh.A[e]);
-    cdf_at(sh.V, e) = cdf_of(sh.V[e]);
-  }
-  __syncthreads();
-  const int ne = n + (n & 1);       // players, with one dummy when n is odd
-  const int np = ne / 2;
-  for (int sweep = 0; sweep < 40; ++sweep) {
-    // convergence: off-diagonal Frobenius norm relative to the whole matrix, at the level
-    // double-float entries resolve (about 2^-46 each)
-    // (in double: the entries of a Gram of tiny columns would underflow when squared in float)
-    double off = 0, tot = 0;
-    for (int e = tid; e < n * n; e += nt) {
-      const CDF a = cdf_at(sh.A, e);
-      const double v = (double)a.re.h * a.re.h + (double)a.im.h * a.im.h;
-      tot += v;
-      if (e / n != e % n) off += v;
-    }
-    off = block_sum(off, sh.red);
-    tot = block_sum(tot, sh.red);
-    if (off <= 1e-25 * tot || off == 0.0) break;
-    if (tid == 0) sh.rot = 0;
-    __syncthreads();
-    for (int round = 0; round < ne - 1; ++round) {
-      if (tid < np) {
-        const int k = tid;
-        const int posa = k, posb = ne - 1 - k;
-        const int p = posa == 0 ? 0 : ((posa - 1 + round) % (ne - 1)) + 1;
-        const int q = ((posb - 1 + round) % (ne - 1)) + 1;
-        // rotation annihilating a_pq, stored as float pairs for the row and column updates.
-        // The angle t = tan(theta) only needs to be close (a rotation by a slightly wrong
-        // angle leaves a tiny a_pq for the next sweep), so it is taken in FP32; c, s and the
-        // unit phase e^{-i phi} must be orthonormal to working precision and are formed in
-        // FP64 from that t (double-float arithmetic would leave c^2 + s^2 - 1 near 1.5e-14,
-        // four times the FP64 rounding, which stalled the 32^4 solves). This keeps the chain
-        // of dependent FP64 operations per round short: it is the latency of every round.
-        double c = 1.0, s = 0.0;
-        double2 eph = make_double2(1.0, 0.0);   // e^{-i phi}
-        int pp = p < q ? p : q, qq = p < q ? q : p;
-        if (qq < n) {
-          const double2 apq = dbl_of(cdf_at(sh.A, pp * n + qq));
-          const double r2 = fma(apq.x, apq.x, apq.y * apq.y);
-          const DF ad = cdf_at(sh.A, pp * n + pp).re, bd = cdf_at(sh.A, qq * n + qq).re;
-          const double a = df_dbl(ad), bq = df_dbl(bd);
-          if (r2 > 1e-300 && r2 > 1.6e-27 * fabs(a * bq)) {
-            sh.rot = 1;
-            const double inv_r = rsqrt(r2);
-            eph = make_double2(apq.x * inv_r, -apq.y * inv_r);
-            // tau = (a_qq - a_pp) / (2 |a_pq|) and t in FP32
-            const float tau = (float)((bq - a) * 0.5) * (float)inv_r;
-            const float at = fabsf(tau);
-            float tf = at > 1e15f ? 0.5f / at : 1.f / (at + sqrtf(fmaf(at, at, 1.f)));
-            if (tau < 0.f) tf = -tf;
-            const double t = (double)tf;
-            c = rsqrt(fma(t, t, 1.0));
-            s = t * c;
-          }
-        } else {
-          pp = -1;
-        }
-        sh.rp[k] = pp; sh.rq[k] = qq;
-        const DF cf = df_of(c), sf = df_of(s);
-        const CDF pf = cdf_of(eph);
-        sh.rot_cs[k] = make_float4(cf.h, cf.l, sf.h, sf.l);
-        sh.rot_ph[k] = make_float4(pf.re.h, pf.re.l, pf.im.h, pf.im.l);
-      }
-      __syncthreads();
-      // columns: A <- A J, V <- V J
-      for (int e = tid; e < n * np; e += nt) {
-        const int i = e / np, k = e % np;
-        const int p = sh.rp[k];
-        if (p < 0 || sh.rot_cs[k].z == 0.f) continue;
-        const int q = sh.rq[k];
-        const float4 cs = sh.rot_cs[k], ph = sh.rot_ph[k];
-        const DF c{cs.x, cs.y}, s{cs.z, cs.w};
-        const CDF eph{DF{ph.x, ph.y}, DF{ph.z, ph.w}};
-        {
-          CDF& aip = cdf_at(sh.A, i * n + p);
-          CDF& aiq = cdf_at(sh.A, i * n + q);
-          const CDF t = cdf_mul(aiq, eph);
-          CDF a2, t2;
-          cdf_rot(aip, t, c, s, a2, t2);
-          aip = a2; aiq = t2;
-        }
-        {
-          CDF& vip = cdf_at(sh.V, i * n + p);
-          CDF& viq = cdf_at(sh.V, i * n + q);
-          const CDF t = cdf_mul(viq, eph);
-          CDF a2, t2;
-          cdf_rot(vip, t, c, s, a2, t2);
-          vip = a2; viq = t2;
-        }
-      }
-      __syncthreads();
-      // rows: A <- J^H A. Consecutive threads walk along a row (j fastest): rows start n
-      // entries of 16 B apart, so threads of one column in different rows would share banks.
-      for (int e = tid; e < n * np; e += nt) {
-        const int k = e / n, j = e % n;
-        const int p = sh.rp[k];
-        if (p < 0 || sh.rot_cs[k].z == 0.f) continue;
-        const int q = sh.rq[k];
-        const float4 cs = sh.rot_cs[k], ph = sh.rot_ph[k];
-        const DF c{cs.x, cs.y}, s{cs.z, cs.w};
-        const CDF ephc{DF{ph.x, ph.y}, DF{-ph.z, -ph.w}};   // e^{+i phi}
-        CDF& apj = cdf_at(sh.A, p * n + j);
-        CDF& aqj = cdf_at(sh.A, q * n + j);
-        const CDF t = cdf_mul(aqj, ephc);
-        CDF a2, t2;
-        cdf_rot(apj, t, c, s, a2, t2);
-        apj = a2; aqj = t2;
-      }
-      __syncthreads();
-    }
-    if (sh.rot == 0) break;
-    __syncthreads();
-  }
-  // back to double: eigenvalues on the diagonal, eigenvectors in V
-  for (int e = tid; e < n * n; e += nt) {
-    sh.A[e] = dbl_of(cdf_at(sh.A, e));
-    sh.V[e] = dbl_of(cdf_at(sh.V, e));
-  }
-  __syncthreads();
-  // sort ascending: rank of every eigenvalue (ties by index)
-  for (int i = tid; i < n; i += nt) sh.w2[i] = sh.A[i * n + i].x;
-  __syncthreads();
-  for (int i = tid; i < n; i += nt) {
-    int rank = 0;
-    const double wi = sh.w2[i];
-    for (int j = 0; j < n; ++j) {
-      const double wj = sh.w2[j];
-      rank += (wj < wi) || (wj == wi && j < i);
-    }
-    sh.perm[rank] = i;
-  }
-  __syncthreads();
-  // A (no longer needed) <- V[:, perm], then V <- A
-  for (int e = tid; e < n * n; e += nt) {
-    const int i = e / n, r = e % n;
-    sh.A[e] = sh.V[i * n + sh.perm[r]];
-  }
-  for (int r = tid; r < n; r += nt) sh.w[r] = sh.w2[sh.perm[r]];
-  __syncthreads();
-  for (int e = tid; e < n * n; e += nt) sh.V[e] = sh.A[e];
-  __syncthreads();
-}
-
-// Orthonormalising transform of a block from its Gram matrix (SVQB):
-// D = diag(G)^{-1/2}, D G D = U S U^H, T = D U S^{-1/2} restricted to S > drop * max(S).
-// Columns of T beyond the kept rank are zero and their mask entry is 0.
-__global__ void __launch_bounds__(kSmallThreads)
-svqb_kernel(Batch bt, const double2* G, int b, double drop, double2* T, int* mask, int* status) {
-  extern __shared__ __align__(16) unsigned char raw[];
-  SmallShared& sh = *reinterpret_cast<SmallShared*>(raw);
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int prob = blockIdx.x;
-  if (bt.active && !bt.active[prob]) return;
-  G += (size_t)prob * kCapG;
-  T += (size_t)prob * kCapT;
-  mask += (size_t)prob * kMaxBlock;
-  if (status) status += prob;
-  for (int i = tid; i < b; i += nt) {
-    const double g = G[i * b + i].x;
-    sh.w[i] = g > 1e-300 ? 1.0 / sqrt(g) : 0.0;
-  }
-  __syncthreads();
-  for (int e = tid; e < b * b; e += nt) {
-    const int i = e / b, j = e % b;
-    const double2 g = G[e];
-    sh.A[e] = make_double2(g.x * sh.w[i] * sh.w[j], g.y * sh.w[i] * sh.w[j]);
-  }
-  // keep D while the eigensolver reuses w
-  for (int i = tid; i < b; i += nt) sh.d[i] = sh.w[i];
-  __syncthreads();
-  jacobi_eig(sh, b);
-  const double smax = sh.w[b - 1];
-  for (int e = tid; e < b * b; e += nt) {
-    const int i = e / b, k = e % b;   // T[i][k]; eigenvalues ascending, keep the largest
-    const int col = b - 1 - k;        // output column k <- eigenpair b-1-k (descending)
-    const double sk = sh.w[col];
-    const double di = sh.d[i];
-    double2 t = make_double2(0, 0);
-    if (smax > 0 && sk > drop * smax) {
-      const double f = di / sqrt(sk);
-      const double2 u = sh.V[i * b + col];
-      t = make_double2(u.x * f, u.y * f);
-    }
-    T[e] = t;
-  }
-  for (int k = tid; k < b; k += nt) {
-    const double sk = sh.w[b - 1 - k];
-    mask[k] = (smax > 0 && sk > drop * smax) ? 1 : 0;
-  }
-  if (tid == 0 && status) *status = 0;
-}
-
-// Rayleigh-Ritz on the orthonormal basis S (m columns, `mask` marks the active ones):
-// eigenpairs of the compacted Hermitian A; theta and Cx (m x b) take the lowest b.
-// Cp: Cx with its first x_rows rows zeroed (the W and P parts), orthogonalised against Cx
-// and orthonormalised in the coefficient space, so that S Cp is orthonormal and orthogonal
-// to S Cx; dependent columns are zero with mask_p = 0.
-__global__ void __launch_bounds__(kSmallThreads)
-rr_kernel(Batch bt, const double2* Ain, int m, int b, const int* mask, int x_rows,
-          double* theta, double2* Cx, double2* Cp, int* mask_p, int* status) {
-  extern __shared__ __align__(16) unsigned char raw[];
-  SmallShared& sh = *reinterpret_cast<SmallShared*>(raw);
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int prob = blockIdx.x;
-  if (bt.active && !bt.active[prob]) return;
-  Ain += (size_t)prob * kCapG;
-  mask += (size_t)prob * kMaxSmall;
-  theta += (size_t)prob * kMaxBlock;
-  Cx += (size_t)prob * kCapC;
-  Cp += (size_t)prob * kCapC;
-  mask_p += (size_t)prob * kMaxBlock;
-  status += prob;
-  if (tid == 0) {
-    int na = 0;
-    for (int i = 0; i < m; ++i) if (mask[i]) sh.idx[na++] = i;
-    sh.flag = na;
-  }
-  __syncthreads();
-  const int na = sh.flag;
-  if (na < b) {
-    if (tid == 0) *status = 1;
-    return;
-  }
-  for (int e = tid; e < na * na; e += nt) {
-    const int i = e / na, j = e % na;
-    sh.A[e] = Ain[sh.idx[i] * m + sh.idx[j]];
-  }
-  __syncthreads();
-  jacobi_eig(sh, na);
-  // Cx (m x b): rows of inactive columns are zero
-  for (int e = tid; e < m * b; e += nt) Cx[e] = make_double2(0, 0);
-  __syncthreads();
-  for (int e = tid; e < na * b; e += nt) {
-    const int i = e / b, k = e % b;
-    Cx[sh.idx[i] * b + k] = sh.V[i * na + k];
-  }
-  for (int k = tid; k < b; k += nt) theta[k] = sh.w[k];
-  __syncthreads();
-  __threadfence_block();
-  // Cp: two rounds of (orthogonalise against Cx twice, then orthonormalise). The second
-  // round acts on unit columns, so the rounding left by normalising tiny first-round
-  // columns (norm down to 1e-12) cannot survive as a loss of orthogonality to Cx.
-  for (int rep = 0; rep < 2; ++rep) {
-    for (int e = tid; e < m * b; e += nt) {
-      const double2 c = Cx[e];
-      sh.A[e] = c;
-      sh.B[e] = rep ? Cp[e] : ((e / b) < x_rows ? make_double2(0, 0) : c);
-    }
-    __syncthreads();
-    for (int pass = 0; pass < 2; ++pass) {
-      for (int e = tid; e < b * b; e += nt) {
-        const int r = e / b, c = e % b;
-        double2 s = make_double2(0, 0);
-        for (int i = 0; i < m; ++i) {
-          const double2 t = cmul(cconj(sh.A[i * b + r]), sh.B[i * b + c]);
-          s.x += t.x; s.y += t.y;
-        }
-        sh.V[e] = s;
-      }
-      __syncthreads();
-      for (int e = tid; e < m * b; e += nt) {
-        const int i = e / b, c = e % b;
-        double2 s = make_double2(0, 0);
-        for (int r = 0; r < b; ++r) {
-          const double2 t = cmul(sh.A[i * b + r], sh.V[r * b + c]);
-          s.x += t.x; s.y += t.y;
-        }
-        sh.V[b * b + e] = make_double2(sh.B[e].x - s.x, sh.B[e].y - s.y);
-      }
-      __syncthreads();
-      for (int e = tid; e < m * b; e += nt) sh.B[e] = sh.V[b * b + e];
-      __syncthreads();
-    }
-    // Gram of Cp, then its SVQB transform in the coefficient space
-    for (int e = tid; e < b * b; e += nt) {
-      const int r = e / b, c = e % b;
-      double2 s = make_double2(0, 0);
-      for (int i = 0; i < m; ++i) {
-        const double2 t = cmul(cconj(sh.B[i * b + r]), sh.B[i * b + c]);
-        s.x += t.x; s.y += t.y;
-      }
-      sh.V[b * b + m * b + e] = s;
-    }
-    __syncthreads();
-    for (int e = tid; e < m * b; e += nt) Cp[e] = sh.B[e];
-    for (int e = tid; e < b * b; e += nt) sh.A[e] = sh.V[b * b + m * b + e];
-    __syncthreads();
-    jacobi_eig(sh, b);
-    // keep columns of norm > 1e-12 in the first round, near-unit columns in the second
-    const double keep = rep ? 1e-2 : 1e-24;
-    for (int e = tid; e < b * b; e += nt) {
-      const int i = e / b, k = e % b;
-      const int col = b - 1 - k;
-      const double sk = sh.w[col];
-      double2 t = make_double2(0, 0);
-      if (sk > keep) {
-        const double f = 1.0 / sqrt(sk);
-        const double2 u = sh.V[i * b + col];
-        t = make_double2(u.x * f, u.y * f);
-      }
-      sh.A[e] = t;
-    }
-    for (int k = tid; k < b; k += nt) mask_p[k] = sh.w[b - 1 - k] > keep ? 1 : 0;
-    __syncthreads();
-    for (int e = tid; e < m * b; e += nt) sh.B[e] = Cp[e];
-    __syncthreads();
-    for (int e = tid; e < m * b; e += nt) {
-      const int i = e / b, c = e % b;
-      double2 s = make_double2(0, 0);
-      for (int r = 0; r < b; ++r) {
-        const double2 t = cmul(sh.B[i * b + r], sh.A[r * b + c]);
-        s.x += t.x; s.y += t.y;
-      }
-      Cp[e] = s;
-    }
-    __syncthreads();
-  }
-  if (tid == 0) *status = 0;
-}
-
 template <typename Tin, typename Tout>
 __global__ void convert_kernel(const Tin* in, Tout* out, long long count) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
@@ -983,7 +509,7 @@ iwf_status gram(const Batch& bt, const BlockList& A, const BlockList& B, long lo
 template <typename T>
 iwf_status block_update(const Batch& bt, const BlockList& S, long long N, const double2* C1,
                         const double2* C2, int cstride, int q, void* out1, void* out2,
-                        bool subtract, cudaStream_t s) {
+                        bool subtract, cudaStream_t s, const double* norms) {
   // (the static attribute flags below are per instantiation of T)
   using V2 = typename Cplx<T>::type;
   const int m = S.nb * S.b;
@@ -991,7 +517,7 @@ iwf_status block_update(const Batch& bt, const BlockList& S, long long N, const 
   if (cstride < m * q) return fail(IWF_ERR_ARG, "block_update: coefficient stride too small");
   if (sizeof(T) == 8 && bt.engine == kEngineTensor)
     return update_tc(bt, S, N, C1, C2, cstride, q, reinterpret_cast<double2*>(out1),
-                     reinterpret_cast<double2*>(out2), subtract, bt.err, s);
+                     reinterpret_cast<double2*>(out2), subtract, bt.err, s, norms);
   int g0 = grid_for(N, kUpdRows);
   if (bt.nprob > 1) g0 = std::max(1, std::min(g0, (8 * 152 + bt.nprob - 1) / bt.nprob));
   const dim3 g(g0, bt.nprob);
@@ -1059,34 +585,6 @@ iwf_status residual_precond(const Batch& bt, const void* X, const void* HX, cons
   return IWF_OK;
 }
 
-static iwf_status small_smem_attr(const void* fn) {
-  IWF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)sizeof(SmallShared)));
-  return IWF_OK;
-}
-
-iwf_status svqb_small(const Batch& bt, const double2* G, int b, double drop, double2* T,
-                      int* mask, int* status, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) { IWF_TRY(small_smem_attr((const void*)svqb_kernel)); attr = true; }
-  svqb_kernel<<<bt.nprob, kSmallThreads, sizeof(SmallShared), s>>>(bt, G, b, drop, T, mask, status);
-  IWF_CUDA(cudaGetLastError());
-  count_launch();
-  return IWF_OK;
-}
-
-iwf_status rayleigh_ritz_small(const Batch& bt, const double2* A, int m, int b, const int* mask,
-                               int x_rows, double* theta, double2* Cx, double2* Cp,
-                               int* mask_p, int* status, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) { IWF_TRY(small_smem_attr((const void*)rr_kernel)); attr = true; }
-  rr_kernel<<<bt.nprob, kSmallThreads, sizeof(SmallShared), s>>>(bt, A, m, b, mask, x_rows, theta,
-                                                                 Cx, Cp, mask_p, status);
-  IWF_CUDA(cudaGetLastError());
-  count_launch();
-  return IWF_OK;
-}
-
 template <typename Tin, typename Tout>
 iwf_status convert_block(const void* in, void* out, long long count, cudaStream_t s) {
   convert_kernel<Tin, Tout><<<grid_for(count, 256), 256, 0, s>>>(
@@ -1128,10 +626,10 @@ template iwf_status gram<float>(const Batch&, const BlockList&, const BlockList&
                                 double2*, double2*, int, cudaStream_t, bool);
 template iwf_status block_update<double>(const Batch&, const BlockList&, long long, const double2*,
                                          const double2*, int, int, void*, void*, bool,
-                                         cudaStream_t);
+                                         cudaStream_t, const double*);
 template iwf_status block_update<float>(const Batch&, const BlockList&, long long, const double2*,
                                         const double2*, int, int, void*, void*, bool,
-                                        cudaStream_t);
+                                        cudaStream_t, const double*);
 template iwf_status residual_precond<double>(const Batch&, const void*, const void*, const double*,
                                              const double*, const double*, const double*, void*,
                                              long long, int, double*, int, double*, cudaStream_t);

@@ -1,6 +1,6 @@
 // Tall-skinny block kernels of the eigensolver: Gram products, block updates, the fused
-// residual / preconditioner step, and the one-CTA dense Hermitian eigensolver used for the
-// small Rayleigh-Ritz and orthonormalisation problems.
+// residual / preconditioner step, and the one-CTA dense problems of the Rayleigh-Ritz step and
+// of the orthonormalisation.
 //
 // A block of b vectors of length N is column-major (column j at offset j*N). A "block list"
 // concatenates up to four blocks of equal width b into one logical N x (nb*b) matrix.
@@ -55,7 +55,48 @@ constexpr int kCapG = kMaxSmall * kMaxSmall;
 constexpr int kCapC = kMaxSmall * kMaxBlock;
 constexpr int kCapT = kMaxBlock * kMaxBlock;
 
-// Host-side launchers (defined in blockops.cu).
+// Double-float helpers (the arithmetic is described in blockops.cu).
+// x = hi + lo with integer and FP32 operations only: conversions between double and float,
+// and double arithmetic, issue on the slow FP64 pipe and made the staging of a tile cost as
+// much as its products. hi is x truncated to 24 significant bits (built from x's sign,
+// exponent and top fraction bits); lo is the remaining 29 fraction bits rounded to a float
+// (two exact 23-bit integer-to-float conversions by the 2^23 bias trick and one fma) times
+// the exact power of two 2^(e - 52). |x| < 2^-126 gives (0, 0); below 2^-75 lo is 0.
+__device__ __forceinline__ void split_bits(double x, float& hi, float& lo) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const unsigned int hw = (unsigned int)(b >> 32), lw = (unsigned int)b;
+  const int e = (int)((hw >> 20) & 0x7ffu);          // biased exponent
+  const unsigned int sign = hw & 0x80000000u;
+  if (e < 1023 - 126) { hi = 0.f; lo = 0.f; return; }
+  const unsigned int top23 = ((hw & 0xfffffu) << 3) | (lw >> 29);
+  hi = __uint_as_float(sign | ((unsigned int)(e - 1023 + 127) << 23) | top23);
+  const unsigned int rest = lw & 0x1fffffffu;
+  const float rh = __uint_as_float(0x4B000000u | (rest >> 23)) - 8388608.f;      // exact
+  const float rl = __uint_as_float(0x4B000000u | (rest & 0x7fffffu)) - 8388608.f;  // exact
+  const float r = fmaf(rh, 8388608.f, rl);
+  const int se = e - 1075 + 127;
+  const float scale = se > 0 ? __uint_as_float((unsigned int)se << 23) : 0.f;
+  lo = r * scale;
+  if (sign) lo = -lo;
+}
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+  s = a + b;
+  const float bb = s - a;
+  e = (a - (s - bb)) + (b - bb);
+}
+// (sh, sl) += (xh + xl)(yh + yl), dropping xl*yl (below 2^-48 relative)
+__device__ __forceinline__ void df_mac(float& sh, float& sl, float xh, float xl, float yh, float yl) {
+  const float p = xh * yh;
+  float t = fmaf(xh, yh, -p);                      // exact: xh*yh = p + t
+  t = fmaf(xh, yl, t);
+  t = fmaf(xl, yh, t);
+  float s, e;
+  two_sum(sh, p, s, e);
+  sh = s;
+  sl += e + t;
+}
+
+// Host-side launchers (defined in blockops.cu; the one-CTA dense problems in small.cu).
 // herm: the product is Hermitian (A^H A, or X^H H X for Hermitian H): only the blocks on and
 // above the 24 x 24 block diagonal are formed, the rest are mirrored.
 template <typename T>
@@ -64,10 +105,15 @@ iwf_status gram(const Batch& bt, const BlockList& A, const BlockList& B, long lo
 // out = S C1 (and out2 = S C2 when C2 != nullptr); subtract: out -= S C1 instead.
 // Problem p's coefficient matrices start at C1 + p*cstride (kCapG for Gram outputs,
 // kCapT for SVQB transforms, kCapC for Rayleigh-Ritz coefficients).
+// norms (may be null; nprob x kMaxBlock; subtract with the tensor engine, ignored elsewhere): the
+// columns' norms at entry, up to a moderate factor. Column j of the result is scaled up by the
+// power of two that brings norms[j] near one. That engine resolves a row of S to 2^-56 of its
+// largest entry, so where a block with columns 1e10 apart in norm is orthonormalised, the smallest
+// would carry 1e-6 of noise once normalised; the other engines round relative to each value.
 template <typename T>
 iwf_status block_update(const Batch& bt, const BlockList& S, long long N, const double2* C1,
                         const double2* C2, int cstride, int q, void* out1, void* out2,
-                        bool subtract, cudaStream_t s);
+                        bool subtract, cudaStream_t s, const double* norms = nullptr);
 // R = HX - X diag(theta); W = M R with M_k = h/(h^2 + off2[p]), h = lam_k + shift[p]
 // (Eq. precond, shifted); squared column norms of R -> resid (sqrt'ed).
 template <typename T>
@@ -91,7 +137,7 @@ iwf_status gram_tc(const Batch& bt, const BlockList& A, const BlockList& B, long
                    bool herm);
 iwf_status update_tc(const Batch& bt, const BlockList& S, long long N, const double2* C1,
                      const double2* C2, int cstride, int q, double2* out1, double2* out2,
-                     bool subtract, int* err, cudaStream_t s);
+                     bool subtract, int* err, cudaStream_t s, const double* norms);
 // *flag = 1 (device int) when any of count doubles at x is NaN or infinite, else 0.
 iwf_status any_nonfinite(const double* x, long long count, int* flag, cudaStream_t s);
 // mask[p*kMaxSmall + off + j] = value (or src[p*kMaxBlock + j]) for j < b, every problem.

@@ -6,7 +6,7 @@
 //   W <- W - [X P]([X P]^H W), twice            (classical Gram-Schmidt, reorthogonalised)
 //   W <- W D U S^{-1/2}, twice                   (SVQB; dependent directions dropped)
 //   HW = H W                                      (the FFT apply)
-//   A = S^H [HX HW HP]; A = Y diag(theta) Y^H     (one-CTA Jacobi per problem, FP64)
+//   A = S^H [HX HW HP]; A = Y diag(theta) Y^H     (one CTA per problem, FP64)
 //   X <- S Yx, P <- S Yp with Yp orthonormalised against Yx in the coefficient space, so
 //   that [X P] stays orthonormal without touching the long vectors again.
 // All problems advance in lockstep through the same kernels (problem index in the grid);
@@ -225,7 +225,9 @@ iwf_status run_phase(iwf_plan* p, const ApplyBatch* ab, int b, int nev, int maxi
     for (int pass = 0; pass < 2; ++pass) {
       const BlockList XP = hasP ? blocks({Xa, Pa}, b) : blocks({Xa}, b);
       IWF_TRY(gram<T>(bt, XP, blocks({W}, b), N, sm.G, sm.partial, sm.slots, st));
-      IWF_TRY(block_update<T>(bt, XP, N, sm.G, nullptr, kCapG, b, W, nullptr, true, st));
+      // the first pass also brings W's columns near unit norm (their norms: the residuals')
+      IWF_TRY(block_update<T>(bt, XP, N, sm.G, nullptr, kCapG, b, W, nullptr, true, st,
+                              pass == 0 ? sm.resid : nullptr));
     }
     for (int pass = 0; pass < 2; ++pass) {
       IWF_TRY(gram<T>(bt, blocks({W}, b), blocks({W}, b), N, sm.G, sm.partial, sm.slots, st, true));

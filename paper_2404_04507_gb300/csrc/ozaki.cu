@@ -102,12 +102,6 @@ __device__ __forceinline__ void store_digits8(const double (&v)[8], int maxb, un
 
 using tc::tile_off;
 
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = a + b;
-  const float bb = s - a;
-  e = (a - (s - bb)) + (b - bb);
-}
-
 __device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity) {
   for (long long r = 0; r < kTcSpin; ++r)
     if (tc::bar_try_wait(bar, parity)) return true;
@@ -591,10 +585,17 @@ __device__ __forceinline__ int magic_int(float x, float scale) {
   return __float_as_int(fmaf(x, scale, 12582912.0f)) - 0x4B400000;
 }
 
+// v 2^e, 0 <= e <= 1000; zeros, denormals, NaN and Inf stay
+__device__ __forceinline__ double scale_up(double v, int e) {
+  const int hi = __double2hiint(v), x = (hi >> 20) & 0x7FF;
+  return x == 0 || x == 0x7FF ? v : __hiloint2double(hi + (e << 20), __double2loint(v));
+}
+
 template <int NMMA, bool SUB>
 __global__ void __launch_bounds__(kUpdThreads, 1)
 update_tc_kernel(Batch bt, BlockList S, int m, long long N, const double2* C1, const double2* C2,
-                 int cstride, int q, double2* out1, double2* out2, int nout, int* err) {
+                 int cstride, int q, double2* out1, double2* out2, int nout, const double* norms,
+                 int* err) {
   using Cfg = UpdCfg<NMMA>;
   const int prob = blockIdx.y;
   if (bt.active && !bt.active[prob]) return;
@@ -607,6 +608,7 @@ update_tc_kernel(Batch bt, BlockList S, int m, long long N, const double2* C1, c
   __shared__ int abort_flag;
   __shared__ int rowexp[kRxRing][128];
   __shared__ int colexpB[NMMA];
+  __shared__ int col_up[NMMA / 2];              // SUB: power of two that scales an output column
   __shared__ const double2* scol[kMaxSmall];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const size_t poff = (size_t)prob * bt.pstride;
@@ -633,6 +635,13 @@ update_tc_kernel(Batch bt, BlockList S, int m, long long N, const double2* C1, c
     }
     colexpB[n] = mx;
   }
+  if (SUB)
+    for (int j = threadIdx.x; j < NMMA / 2; j += blockDim.x) {
+      int e = 0;                                // (zero, large or not finite norms: as it is)
+      if (norms && j < q)
+        e = 1022 - ((__double2hiint(norms[(size_t)prob * kMaxBlock + j]) >> 20) & 0x7FF);
+      col_up[j] = e < 0 || e > 1000 ? 0 : e;
+    }
   if (threadIdx.x == 0) {
     for (int sl = 0; sl < kUpdSlots; ++sl) {
       tc::bar_init(tc::smem_u32(&full_bar[sl]), kUpdProd * 32);
@@ -848,7 +857,8 @@ update_tc_kernel(Batch bt, BlockList S, int m, long long N, const double2* C1, c
           double2* dst = Y + (size_t)jc * N + r;
           if (SUB) {
             const double2 old = *dst;
-            *dst = make_double2(old.x - val[0], old.y - val[1]);
+            *dst = make_double2(scale_up(old.x - val[0], col_up[jc]),
+                                scale_up(old.y - val[1], col_up[jc]));
           } else {
             *dst = make_double2(val[0], val[1]);
           }
@@ -920,7 +930,8 @@ iwf_status launch_gram_tc(const Batch& bt, const BlockList& A, const BlockList& 
 template <int NMMA, bool SUB>
 iwf_status launch_update_tc(const Batch& bt, const BlockList& S, int m, long long N,
                             const double2* C1, const double2* C2, int cstride, int q,
-                            double2* out1, double2* out2, int* err, cudaStream_t s) {
+                            double2* out1, double2* out2, int* err, cudaStream_t s,
+                            const double* norms) {
   using Cfg = UpdCfg<NMMA>;
   static bool attr[64] = {};
   int dev = 0;
@@ -936,7 +947,7 @@ iwf_status launch_update_tc(const Batch& bt, const BlockList& S, int m, long lon
   slots = std::min(slots, ntiles);
   dim3 grid((unsigned)(slots * nout), (unsigned)bt.nprob);
   update_tc_kernel<NMMA, SUB><<<grid, kUpdThreads, Cfg::kSmem, s>>>(bt, S, m, N, C1, C2, cstride,
-                                                                    q, out1, out2, nout, err);
+                                                                    q, out1, out2, nout, norms, err);
   IWF_CUDA(cudaGetLastError());
   count_launch();
   return IWF_OK;
@@ -992,7 +1003,7 @@ iwf_status gram_tc(const Batch& bt, const BlockList& A, const BlockList& B, long
 
 iwf_status update_tc(const Batch& bt, const BlockList& S, long long N, const double2* C1,
                      const double2* C2, int cstride, int q, double2* out1, double2* out2,
-                     bool subtract, int* err, cudaStream_t s) {
+                     bool subtract, int* err, cudaStream_t s, const double* norms) {
   const int m = S.nb * S.b;
   if (m > kMaxSmall || q < 1 || q > kMaxBlock) return fail(IWF_ERR_ARG, "update_tc: shape");
   const int nm = ((2 * q + 15) / 16) * 16;
@@ -1000,8 +1011,9 @@ iwf_status update_tc(const Batch& bt, const BlockList& S, long long N, const dou
   if (nm == NM) {                                                                          \
     if (subtract)                                                                          \
       return launch_update_tc<NM, true>(bt, S, m, N, C1, nullptr, cstride, q, out1, nullptr, \
-                                        err, s);                                           \
-    return launch_update_tc<NM, false>(bt, S, m, N, C1, C2, cstride, q, out1, out2, err, s); \
+                                        err, s, norms);                                    \
+    return launch_update_tc<NM, false>(bt, S, m, N, C1, C2, cstride, q, out1, out2, err, s, \
+                                       nullptr);                                           \
   }
   IWF_UPD(16) IWF_UPD(32) IWF_UPD(48)
 #undef IWF_UPD
