@@ -132,7 +132,11 @@ iwf_status iwf_set_potential(iwf_plan* plan, int nmodes, const int* m, const dou
 /*
  * hpsi = H~ psi = Lambda psi + F V F^{-1} psi for nvec vectors (Sec. 4.1, Eq. pseudospectral
  * vector), with F = T F* (Sec. 3.3, Eq. F): gather through the index shift, inverse n-D
- * FFT, multiply by V, forward n-D FFT, scatter back to the window and add Lambda psi.
+ * FFT, multiply by V, forward n-D FFT, scatter back to the window and add Lambda psi. With
+ * IWF_PATH_AUTO (the default) and a potential of few folded modes (complex double: at most 24,
+ * or 48 with real coefficients; complex float: 20) the same operator is applied as a direct
+ * convolution with the modes, as iwf_apply_stencil does: one pass, no workspace. A NaN or Inf
+ * in psi then reaches the neighbouring coefficients instead of the whole vector.
  *   precision  IWF_PREC_F64 (complex double I/O and arithmetic) or IWF_PREC_C64
  *              (complex float I/O and arithmetic, Lambda applied in float).
  *   psi, hpsi  device, N*nvec elements each, column-major, window order; must not overlap.
@@ -324,7 +328,8 @@ iwf_status iwf_ws_phase(const iwf_plan* plan, int nprob, int nvec, const double*
                         int sign, void* vecs, void* stream);
 
 /*
- * Same computation as iwf_apply, with CUDA events recorded on `stream` around every pass
+ * H~ psi by the transforms (never the direct convolution that iwf_apply may take), with CUDA
+ * events recorded on `stream` around every pass
  * kernel (pass A: inverse DFT along k_I with the gather; pass B: k_II inverse DFT, V,
  * k_II forward DFT; pass C: forward DFT along k_I with the scatter and Lambda psi).
  * Synchronises the stream. Host outputs (may be NULL): pass_ms[3] = summed device time of
@@ -418,7 +423,7 @@ iwf_status iwf_field_distance(iwf_plan* plan, const void* u, const void* v, long
 /*
  * H~ psi by direct convolution instead of the FFT passes: Lambda psi + sum_m Vg_m psi(k* - m),
  * the cyclic convolution on the K* grid with the potential's folded modes that F V F^{-1}
- * equals (Sec. 3.3, Sec. 4.1, App. C). An ablation for potentials with few modes (at most
+ * equals (Sec. 3.3, Sec. 4.1, App. C). For potentials with few modes (at most
  * 256 folded modes, else IWF_ERR_UNSUPPORTED; fastest k_I axis at most 32): its cost per
  * point grows with the number of modes, the FFT passes' does not. Same arguments, layout and
  * results (up to rounding) as iwf_apply; enqueues on `stream`.
@@ -434,7 +439,8 @@ iwf_status iwf_apply_stencil(iwf_plan* plan, int precision, const void* psi, voi
  *   IWF_PATH_PENCIL  keeps one pencil per thread in registers, loaded from and stored to
  *                    global memory directly, with one shared-memory transpose per pass;
  *                    needs n = 4, d = 2 with 2K_1 = 2K_2 and 2L_1 = 2L_2, each 16 or 32;
- *   IWF_PATH_AUTO    the pencil path where the geometry allows it, else the tiled path.
+ *   IWF_PATH_AUTO    the direct convolution for potentials with few modes (iwf_apply); else
+ *                    the pencil path where the geometry allows it, else the tiled path.
  */
 enum { IWF_PATH_AUTO = 0, IWF_PATH_TILED = 1, IWF_PATH_PENCIL = 2 };
 
@@ -443,8 +449,10 @@ enum { IWF_PATH_AUTO = 0, IWF_PATH_TILED = 1, IWF_PATH_PENCIL = 2 };
  * freed by the call) for every candidate schedule and keeps the fastest for this plan and
  * precision. Candidates: the tiled path with threads per CTA {128, 256}, shared-memory tile
  * budget {24, 48, 96, 160} KB and L2 chunk of vectors between passes {24, 48, 96} MB; where
- * the geometry allows it, the pencil path with chunks {12, 24, 48, 96} MB. Host outputs
- * (may be NULL): *best_ms per apply, best[3] = {threads, tile_kb, chunk_mb} (threads and
+ * the geometry allows it, the pencil path with chunks {12, 24, 48, 96} MB. On a plan whose path
+ * is IWF_PATH_AUTO the direct convolution takes part where the potential allows it; when it
+ * wins the path stays IWF_PATH_AUTO, with the best schedule of the transforms kept for other
+ * potentials. Host outputs (may be NULL): *best_ms per apply, best[3] = {threads, tile_kb, chunk_mb} (threads and
  * tile_kb are 0 when the pencil path won; iwf_plan_get_schedule reports the path). Needs a
  * potential. Results are identical for every schedule up to floating-point summation order;
  * synchronises.

@@ -14,6 +14,8 @@
 // L = 20) runs as per-axis passes: inverse DFTs along its slower axes one at a time (KIND 0
 // on a one-axis group), the last axis with the multiply by V as pass B, then the forward DFTs
 // back along the slower axes (KIND 3).
+// Potentials with few modes need no transform: iwf_apply takes the direct convolution of
+// stencil.cu for them (direct_pays).
 // Rolls are index permutations inside a pencil and cost no arithmetic. Vectors are processed
 // in chunks sized so that the intermediate block stays resident in the 129 MB L2.
 //
@@ -987,21 +989,29 @@ iwf_status stop_timer(PassTimer* timer, int kind, cudaStream_t stream) {
   return IWF_OK;
 }
 
+// Shared-memory bytes of a pass's tile (*tbytes) and of its CTA (*bytes); refuses groups whose
+// smallest tile does not fit.
+template <typename T, int KIND>
+iwf_status pass_smem(const PassArgs& a, size_t* tbytes, size_t* bytes) {
+  const size_t elems = (size_t)a.Ot * a.M * a.C;
+  *tbytes = ((elems + elems / 32 + 1) * sizeof(typename Vec2<T>::type) + 15) / 16 * 16;
+  *bytes = *tbytes + (KIND == 1 ? (size_t)(a.M + a.C) * sizeof(T) : 0);
+  if (*bytes > 200 * 1024) return fail(IWF_ERR_UNSUPPORTED, "apply: tile exceeds shared memory");
+  const int vmin = long_group_values(a);
+  if (vmin > 0 && elems > (size_t)vmin * kLongThreads)
+    return fail(IWF_ERR_UNSUPPORTED, "apply: axis group too large for the shared-memory FFT");
+  return IWF_OK;
+}
+
 // tkind: the pass (0 A, 1 B, 2 C) whose time the launch counts toward (-1: its own KIND)
 template <typename T, int KIND>
 iwf_status launch_pass(PassArgs a, int nvec, cudaStream_t stream, PassTimer* timer, int threads,
                        int tkind = -1) {
-  const size_t elems = (size_t)a.Ot * a.M * a.C;
-  const size_t tbytes = ((elems + elems / 32 + 1) * sizeof(typename Vec2<T>::type) + 15) / 16 * 16;
+  size_t tbytes = 0, bytes = 0;
+  IWF_TRY((pass_smem<T, KIND>(a, &tbytes, &bytes)));
   a.tile_bytes = (int)tbytes;
-  const size_t bytes = tbytes + (KIND == 1 ? (size_t)(a.M + a.C) * sizeof(T) : 0);
-  if (bytes > 200 * 1024) return fail(IWF_ERR_UNSUPPORTED, "apply: tile exceeds shared memory");
   const int vmin = long_group_values(a);
-  if (vmin > 0) {
-    threads = kLongThreads;
-    if (elems > (size_t)vmin * kLongThreads)
-      return fail(IWF_ERR_UNSUPPORTED, "apply: axis group too large for the shared-memory FFT");
-  }
+  if (vmin > 0) threads = kLongThreads;
   static bool attr_set[2][4][2] = {};
   const int ti = sizeof(T) == 8 ? 0 : 1;
   const int li = vmin > 0 ? 1 : 0;
@@ -1167,6 +1177,23 @@ iwf_status pencil_chunk(PencilArgs a, int LI, int LII, const void* in, void* wk,
                   : launch_pencil_ac<T, 32, 2, U>(a, nv, err, stream, timer);
 }
 
+// Whether the direct convolution (stencil.cu) runs the apply: its cost grows with the modes, the
+// transforms' does not. The limits lie where the fastest transforms (pencil set) were overtaken
+// on no window measured. Microseconds of transforms against direct, 16 vectors at 32^4 and (in
+// parentheses) 16^4: complex double 4330 (213), 24 complex modes 2669 (179), 32 3527 (235),
+// 48 real modes 2672 (179); complex float 184 (20), 16 complex modes 132 (15), 24 178 (19),
+// 32 225 (22). The tiled set is slower than the pencil set on every window (22^4, 24 vectors:
+// 5580 and 381 us; direct with 8 complex modes 356 and 36).
+template <typename T>
+bool direct_pays(const iwf_plan* p, const ApplyBatch* batch) {
+  if (p->path[sizeof(T) == 8 ? 0 : 1] != IWF_PATH_AUTO) return false;
+  if (sizeof(T) == 8 && p->fft_arith != IWF_ARITH_F64) return false;
+  if (batch && !batch->modes) return false;
+  const int nm = batch ? batch->nm : p->stencil_nm;
+  const bool real = batch ? batch->real : p->stencil_real;
+  return nm <= (sizeof(T) == 8 ? (real ? 48 : 24) : 20);
+}
+
 template <typename T>
 iwf_status apply_typed(iwf_plan* p, const void* psi, void* hpsi, int nvec, cudaStream_t stream,
                        PassTimer* timer, void* ext_work = nullptr, size_t ext_bytes = 0,
@@ -1182,14 +1209,10 @@ iwf_status apply_typed(iwf_plan* p, const void* psi, void* hpsi, int nvec, cudaS
   if (chunk < 1) chunk = 1;
   if (chunk > nvec) chunk = nvec;
   if (chunk > 65535) chunk = 65535;
-  void* work = ext_work;
   if (ext_work) {
     const int fit = (int)(ext_bytes / vbytes);
     if (fit < 1) return fail(IWF_ERR_UNSUPPORTED, "caller workspace smaller than one vector");
     if (chunk > fit) chunk = fit;
-  } else {
-    IWF_TRY(ensure_workspace(p, vbytes * chunk));
-    work = p->d_work;
   }
 
   PotDev pot{};
@@ -1257,6 +1280,21 @@ iwf_status apply_typed(iwf_plan* p, const void* psi, void* hpsi, int nvec, cudaS
     }
   } else {
     choose_tile<T>(B, tile_kb);
+  }
+
+  // potentials with few modes need no transform; the geometries the passes refuse stay refused
+  if (!timer && direct_pays<T>(p, batch)) {
+    size_t tb, sb;
+    IWF_TRY((pass_smem<T, 0>(A, &tb, &sb)));
+    if (!split) IWF_TRY((pass_smem<T, 1>(B, &tb, &sb)));
+    for (int j = 0; split && j < n - d; ++j) IWF_TRY((pass_smem<T, 1>(Bs[j], &tb, &sb)));
+    return apply_direct(p, sizeof(T) == 8 ? IWF_PREC_F64 : IWF_PREC_C64, psi, hpsi, nvec, stream, batch);
+  }
+
+  void* work = ext_work;
+  if (!ext_work) {
+    IWF_TRY(ensure_workspace(p, vbytes * chunk));
+    work = p->d_work;
   }
 
   PassArgs Cp = A;
@@ -1371,6 +1409,7 @@ iwf_status autotune_impl(iwf_plan* p, int precision, int nvec, double* best_ms, 
   double best_t = 1e30;
   int bt = p->tune_threads[ti], bk = p->tune_tile_kb[ti], bc = p->tune_chunk_mb[ti];
   int bp = IWF_PATH_TILED;
+  double direct_t = 1e30;
   const int saved_path = p->path[ti];
   iwf_status st = IWF_OK;
   // times one candidate (the plan already holds it); keeps it if it is the fastest so far
@@ -1386,7 +1425,8 @@ iwf_status autotune_impl(iwf_plan* p, int precision, int nvec, double* best_ms, 
     if (cudaEventSynchronize(e1) != cudaSuccess) { st = fail(IWF_ERR_CUDA, "autotune timing"); return; }
     float ms = 0.f;
     cudaEventElapsedTime(&ms, e0, e1);
-    if (ms / 3 < best_t) { best_t = ms / 3; bt = th; bk = tk; bc = ch; bp = path; }
+    if (path == IWF_PATH_AUTO) direct_t = ms / 3;
+    else if (ms / 3 < best_t) { best_t = ms / 3; bt = th; bk = tk; bc = ch; bp = path; }
   };
   // double-float DFTs exist on the pencil path only: no tiled candidates then
   const bool df_only = precision == IWF_PREC_F64 && p->fft_arith == IWF_ARITH_DF;
@@ -1397,14 +1437,21 @@ iwf_status autotune_impl(iwf_plan* p, int precision, int nvec, double* best_ms, 
   int LI = 0, LII = 0;
   if (saved_path != IWF_PATH_TILED && pencil_geometry(p->g, &LI, &LII))
     for (int ch : pencil_chunks) trial(IWF_PATH_PENCIL, p->tune_threads[ti], p->tune_tile_kb[ti], ch);
+  // IWF_PATH_AUTO also stands for the direct apply, where the potential has few enough modes
+  p->path[ti] = saved_path;
+  const bool direct = saved_path == IWF_PATH_AUTO &&
+                      (ti == 0 ? direct_pays<double>(p, nullptr) : direct_pays<float>(p, nullptr));
+  if (direct) trial(IWF_PATH_AUTO, bt, bk, bc);
   p->tune_threads[ti] = bt; p->tune_tile_kb[ti] = bk; p->tune_chunk_mb[ti] = bc;
-  p->path[ti] = bp;
+  const int natural = pencil_geometry(p->g, &LI, &LII) ? IWF_PATH_PENCIL : IWF_PATH_TILED;
+  p->path[ti] = saved_path == IWF_PATH_AUTO && (direct ? direct_t < best_t : bp == natural)
+                    ? IWF_PATH_AUTO : bp;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   cudaFree(x);
   cudaFree(y);
   if (st != IWF_OK) { p->path[ti] = saved_path; return st; }
-  if (best_ms) *best_ms = best_t;
+  if (best_ms) *best_ms = p->path[ti] == IWF_PATH_AUTO ? std::fmin(best_t, direct_t) : best_t;
   if (best) {
     best[0] = bp == IWF_PATH_PENCIL ? 0 : bt;
     best[1] = bp == IWF_PATH_PENCIL ? 0 : bk;

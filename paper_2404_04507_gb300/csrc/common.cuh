@@ -114,6 +114,14 @@ struct ApplyBatch {
   long long tab_stride;
   int vecs_per_prob;
   const int* active;
+  // the problems' folded modes for the direct apply: one list of nm shifts for all of them
+  // (device, nm x n, without the constant; null: too many), their coefficients (nprob x nm, 0
+  // where a problem has no such mode) and constant terms (nprob)
+  const int* modes;
+  const double2* coef;
+  const double* cst;
+  int nm;
+  bool real;               // every coefficient is real
 };
 
 }  // namespace iwf
@@ -142,11 +150,15 @@ struct iwf_plan {
   double voff_abs = 0.0;                  // sum_{m != 0} |Vg_m|
   double voff_sq = 0.0;                   // sum_{m != 0} |Vg_m|^2
   int tab_off[IWF_MAX_N] = {};
-  // folded modes of the potential for the direct-convolution apply (iwf_apply_stencil):
-  // stencil_m[q*n + j] in [0, lens[j]), coefficient stencil_c[q] = Vg (re, im)
+  // folded modes of the potential for the direct-convolution apply, without the constant term
+  // (vconst): stencil_m[q*n + j] in [0, lens[j]), coefficient stencil_c[q] = Vg (re, im)
   int stencil_nm = 0;
+  bool stencil_const = false;             // the potential has a constant term
+  bool stencil_real = false;              // every coefficient is real
   int* d_stencil_m = nullptr;
   double2* d_stencil_c = nullptr;
+  std::vector<int> h_stencil_m;           // host copies, for batches of plans
+  std::vector<double2> h_stencil_c;
   // exp(2 pi i j / len), j < len, for every axis of a group with an axis longer than
   // IWF_MAX_LEN (null otherwise)
   double2* d_ltw64[IWF_MAX_N] = {};
@@ -197,6 +209,9 @@ iwf_status apply_noalloc_impl(iwf_plan* p, int precision, const void* psi, void*
                               cudaStream_t stream);
 iwf_status apply_host_impl(iwf_plan* p, int precision, const void* psi_host, void* hpsi_host,
                            int nvec, cudaStream_t stream);
+// The direct apply without argument checks (the caller's), of a plan's potential or a batch's.
+iwf_status apply_direct(const iwf_plan* p, int precision, const void* psi, void* hpsi, int nvec,
+                        cudaStream_t stream, const ApplyBatch* batch);
 iwf_status apply_stencil_impl(iwf_plan* p, int precision, const void* psi, void* hpsi, int nvec,
                               cudaStream_t stream);
 iwf_status evaluate_impl(iwf_plan* p, const void* coef, const double* x, long long M,
@@ -240,6 +255,8 @@ iwf_status build_potential(iwf_plan* p, int nmodes, const int* m, const double* 
 struct PotSummary {
   double vg0 = 0, off_abs = 0, off_sq = 0;
   bool separable = true;
+  std::vector<int> m;              // folded modes without the constant, n ints each
+  std::vector<double2> coef;
 };
 // Per-axis tables (scaled by 1/N, constant folded into axis 0) of one separable potential,
 // written at tab64/tab32 (length sum of lens); the host summary goes to *sum.

@@ -527,6 +527,59 @@ iwf_status check_opts(const iwf_plan* p, const iwf_solve_opts* o) {
   return IWF_OK;
 }
 
+// The direct-apply modes of a batch: the union of the problems' shifts, with every problem's
+// coefficients (0 where it has no such mode) and constant. Leaves ab.modes null when the union
+// is longer than any list the direct apply would take.
+constexpr int kMaxBatchModes = 64;
+struct BatchModes {
+  std::vector<int> m;
+  std::vector<std::vector<double2>> coef;   // per problem, as long as the union was then
+  std::vector<double> cst;
+  void add(int n, const std::vector<int>& pm, const std::vector<double2>& pc, double c0) {
+    coef.emplace_back(m.size() / n, make_double2(0.0, 0.0));
+    cst.push_back(c0);
+    std::vector<double2>& c = coef.back();
+    for (size_t q = 0; q < pc.size() && m.size() <= (size_t)kMaxBatchModes * n; ++q) {
+      size_t r = 0;
+      while (r < c.size() && !std::equal(m.begin() + r * n, m.begin() + (r + 1) * n, pm.begin() + q * n)) ++r;
+      if (r == c.size()) {
+        m.insert(m.end(), pm.begin() + q * n, pm.begin() + (q + 1) * n);
+        c.push_back(make_double2(0.0, 0.0));
+      }
+      c[r] = pc[q];
+    }
+  }
+  iwf_status upload(int n, Arena& ar, ApplyBatch& ab, cudaStream_t s) {
+    const size_t nm = m.size() / n, np = coef.size();
+    ab.modes = nullptr;
+    int* dm;
+    double2* dc;
+    double* d0;
+    // requested either way: the workspace sequence stays fixed
+    IWF_TRY(ar.get(&dm, (size_t)kMaxBatchModes * IWF_MAX_N));
+    IWF_TRY(ar.get(&dc, np * kMaxBatchModes));
+    IWF_TRY(ar.get(&d0, np));
+    if (nm > kMaxBatchModes) return IWF_OK;
+    std::vector<double2> flat(std::max<size_t>(1, np * nm), make_double2(0.0, 0.0));
+    bool real = true;
+    for (size_t q = 0; q < np; ++q)
+      for (size_t r = 0; r < coef[q].size(); ++r) {
+        flat[q * nm + r] = coef[q][r];
+        real = real && coef[q][r].y == 0.0;
+      }
+    IWF_CUDA(cudaMemcpyAsync(dm, m.data(), sizeof(int) * m.size(), cudaMemcpyHostToDevice, s));
+    IWF_CUDA(cudaMemcpyAsync(dc, flat.data(), sizeof(double2) * np * nm, cudaMemcpyHostToDevice, s));
+    IWF_CUDA(cudaMemcpyAsync(d0, cst.data(), sizeof(double) * np, cudaMemcpyHostToDevice, s));
+    IWF_CUDA(cudaStreamSynchronize(s));       // the host copies go out of scope
+    ab.modes = dm;
+    ab.coef = dc;
+    ab.cst = d0;
+    ab.nm = (int)nm;
+    ab.real = real;
+    return IWF_OK;
+  }
+};
+
 // The solve runs on a library stream ordered after the caller's stream (so it can be
 // captured into graphs whatever stream the caller uses).
 struct SolveStream {
@@ -586,6 +639,7 @@ iwf_status batch_eigensolve_impl(iwf_plan* p, int nprob, const int* nmodes, cons
   IWF_TRY(ar.get(&tab32, (size_t)nprob * stride));
   std::vector<double> shift(nprob), off2(nprob);
   long long mo = 0;
+  BatchModes bm;
   for (int q = 0; q < nprob; ++q) {
     if (nmodes[q] < 0 || (nmodes[q] > 0 && (!m || !re || !im)))
       return fail(IWF_ERR_ARG, "iwf_batch_eigensolve: bad mode list");
@@ -595,11 +649,13 @@ iwf_status batch_eigensolve_impl(iwf_plan* p, int nprob, const int* nmodes, cons
     const double sigma = s.off_abs - s.vg0 + 1.0;
     shift[q] = s.vg0 + sigma;
     off2[q] = s.off_sq;
+    bm.add(p->g.n, s.m, s.coef, s.vg0);
     mo += nmodes[q];
   }
   IWF_CUDA(cudaMemcpyAsync(sm.shift, shift.data(), sizeof(double) * nprob, cudaMemcpyHostToDevice, ss.s));
   IWF_CUDA(cudaMemcpyAsync(sm.off2, off2.data(), sizeof(double) * nprob, cudaMemcpyHostToDevice, ss.s));
   ApplyBatch ab{tab64, tab32, stride, b, sm.active};
+  IWF_TRY(bm.upload(p->g.n, ar, ab, ss.s));
   return solve_problems(p, &ab, o, sm, ar, X0, evals, evecs, resid, iters, info, ss.s);
 }
 
@@ -652,6 +708,7 @@ iwf_status run_group(iwf_plan* const* plans, GroupJob& job, const iwf_solve_opts
   // apply's convention), and its preconditioner parameters
   std::vector<double> t64((size_t)np * stride), shift(np), off2(np);
   std::vector<float> t32((size_t)np * stride);
+  BatchModes bm;
   for (int q = 0; q < np; ++q) {
     const iwf_plan* p = plans[job.idx[q]];
     IWF_CUDA(cudaMemcpy(t64.data() + (size_t)q * stride, p->d_tab64, sizeof(double) * stride,
@@ -661,6 +718,7 @@ iwf_status run_group(iwf_plan* const* plans, GroupJob& job, const iwf_solve_opts
     const double sigma = p->voff_abs - p->vg0 + 1.0;
     shift[q] = p->vg0 + sigma;
     off2[q] = p->voff_sq;
+    bm.add(gp->g.n, p->h_stencil_m, p->h_stencil_c, p->vconst);
   }
   for (size_t i = 0; i < t64.size(); ++i) t32[i] = (float)t64[i];
   IWF_CUDA(cudaMemcpyAsync(tab64, t64.data(), sizeof(double) * t64.size(), cudaMemcpyHostToDevice, ss.s));
@@ -687,6 +745,7 @@ iwf_status run_group(iwf_plan* const* plans, GroupJob& job, const iwf_solve_opts
   std::vector<double> ev((size_t)np * nev), rs((size_t)np * nev);
   std::vector<int> it(np);
   ApplyBatch ab{tab64, tab32, stride, b, sm.active};
+  IWF_TRY(bm.upload(gp->g.n, ar, ab, ss.s));
   const iwf_status st = solve_problems(gp, &ab, o, sm, ar, X0cat, ev.data(), V, rs.data(),
                                        it.data(), &job.info, ss.s);
   if (st != IWF_OK && st != IWF_ERR_NOCONV) return st;

@@ -289,6 +289,17 @@ iwf_status fold_modes(const Geom& g, int nmodes, const int* m, const double* re,
   }
   return IWF_OK;
 }
+
+// The folded modes without the constant term, as the direct apply takes them.
+void direct_modes(const Folded& F, int n, std::vector<int>& m, std::vector<double2>& coef) {
+  m.clear();
+  coef.clear();
+  for (size_t q = 0; q < F.re.size(); ++q) {
+    if (F.axis[q] == -1) continue;
+    m.insert(m.end(), F.m.begin() + q * n, F.m.begin() + (q + 1) * n);
+    coef.push_back(make_double2(F.re[q], F.im[q]));
+  }
+}
 }  // namespace
 
 iwf_status build_potential(iwf_plan* p, int nmodes, const int* m, const double* re,
@@ -356,15 +367,18 @@ iwf_status build_potential(iwf_plan* p, int nmodes, const int* m, const double* 
   p->d_stencil_m = nullptr;
   p->d_stencil_c = nullptr;
   p->stencil_nm = 0;
-  if (nm) {
-    std::vector<double2> coef(nm);
-    for (size_t q = 0; q < nm; ++q) coef[q] = make_double2(fre[q], fim[q]);
-    IWF_CUDA(cudaMalloc((void**)&p->d_stencil_m, nm * n * sizeof(int)));
-    IWF_CUDA(cudaMalloc((void**)&p->d_stencil_c, nm * sizeof(double2)));
-    IWF_CUDA(cudaMemcpy(p->d_stencil_m, fm.data(), nm * n * sizeof(int), cudaMemcpyHostToDevice));
-    IWF_CUDA(cudaMemcpy(p->d_stencil_c, coef.data(), nm * sizeof(double2), cudaMemcpyHostToDevice));
+  direct_modes(F, n, p->h_stencil_m, p->h_stencil_c);
+  p->stencil_const = p->h_stencil_c.size() < nm;
+  p->stencil_real = true;
+  for (const double2& c : p->h_stencil_c) p->stencil_real = p->stencil_real && c.y == 0.0;
+  const size_t nd = p->h_stencil_c.size();
+  if (nd) {
+    IWF_CUDA(cudaMalloc((void**)&p->d_stencil_m, nd * n * sizeof(int)));
+    IWF_CUDA(cudaMalloc((void**)&p->d_stencil_c, nd * sizeof(double2)));
+    IWF_CUDA(cudaMemcpy(p->d_stencil_m, p->h_stencil_m.data(), nd * n * sizeof(int), cudaMemcpyHostToDevice));
+    IWF_CUDA(cudaMemcpy(p->d_stencil_c, p->h_stencil_c.data(), nd * sizeof(double2), cudaMemcpyHostToDevice));
   }
-  p->stencil_nm = (int)nm;
+  p->stencil_nm = (int)nd;
   IWF_CUDA(cudaDeviceSynchronize());
   return IWF_OK;
 }
@@ -380,6 +394,7 @@ iwf_status potential_tables(const iwf_plan* p, int nmodes, const int* m, const d
     return fail(IWF_ERR_UNSUPPORTED, "batched solves need potentials whose modes each lie on one "
                                      "lifted axis");
   sum->vg0 = F.vg0; sum->off_abs = F.off_abs; sum->off_sq = F.off_sq; sum->separable = true;
+  direct_modes(F, n, sum->m, sum->coef);
   const size_t nm = F.re.size();
   std::vector<int> tax, tl;
   int total = 0;
