@@ -11,6 +11,7 @@ namespace {
 constexpr int kGramRows = 16;      // rows staged per Gram tile
 constexpr int kGramTx = 24;        // 24 x 24 threads, 3 x 3 outputs each -> up to 72 x 72
 constexpr int kGramThreads = kGramTx * kGramTx;
+constexpr int kRedWarps = 8;       // warps that share the slots of a reduction
 
 template <typename T> struct Acc { using type = double; };
 template <> struct Acc<float> { using type = float; };
@@ -192,27 +193,35 @@ gram_df_kernel(Batch bt, BlockList A, BlockList B, int ma, int mb, long long N, 
     }
 }
 
-// Sum the per-CTA partials in a fixed order (deterministic); problem blockIdx.y.
+// Sum the per-CTA partials in a fixed order (deterministic); problem blockIdx.y. A CTA takes 32
+// entries, its eight warps every eighth slot each: one thread an entry walked 608 slots one FP64
+// addition after another (130 us at 72 x 72).
 // herm: entries in 24 x 24 blocks below the block diagonal were not formed; they are the
 // conjugates of their mirror images (mb = row length).
 __global__ void reduce_partials(Batch bt, const double2* partial, int slots, int count,
                                 double2* out, bool herm, int mb) {
   const int prob = blockIdx.y;
   if (bt.active && !bt.active[prob]) return;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= count) return;
-  int src = e;
+  __shared__ double2 part[kRedWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + lane;
+  const bool live = e < count;
+  int src = live ? e : 0;
   bool conj = false;
-  if (herm) {
+  if (herm && live) {
     const int a = e / mb, c = e % mb;
     if (a / kGramTx > c / kGramTx) { src = c * mb + a; conj = true; }
   }
   const double2* pp = partial + (size_t)prob * slots * count;
   double re = 0, im = 0;
-  for (int s = 0; s < slots; ++s) {
+  for (int s = warp; s < slots; s += kRedWarps) {
     const double2 v = pp[(size_t)s * count + src];
     re += v.x; im += v.y;
   }
+  part[warp][lane] = make_double2(re, im);
+  __syncthreads();
+  if (warp > 0 || !live) return;
+  for (int w = 1; w < kRedWarps; ++w) { re += part[w][lane].x; im += part[w][lane].y; }
   out[(size_t)prob * kCapG + e] = make_double2(re, conj ? -im : im);
 }
 
@@ -407,13 +416,18 @@ residual_kernel(Batch bt, const typename Cplx<T>::type* X, const typename Cplx<T
   }
 }
 
+// One CTA a problem: lane j sums column j, its warps every kRedWarps-th slot.
 __global__ void resid_finish(Batch bt, const double* partial, int slots, int b, double* resid) {
   const int prob = blockIdx.x;
   if (bt.active && !bt.active[prob]) return;
-  const int j = threadIdx.x;
-  if (j >= b) return;
+  __shared__ double part[kRedWarps][32];
+  const int j = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double s = 0;
-  for (int c = 0; c < slots; ++c) s += partial[((size_t)prob * slots + c) * b + j];
+  for (int c = warp; j < b && c < slots; c += kRedWarps) s += partial[((size_t)prob * slots + c) * b + j];
+  part[warp][j] = s;
+  __syncthreads();
+  if (warp > 0 || j >= b) return;
+  for (int w = 1; w < kRedWarps; ++w) s += part[w][j];
   resid[(size_t)prob * kMaxBlock + j] = sqrt(s);
 }
 
@@ -479,8 +493,11 @@ iwf_status gram(const Batch& bt, const BlockList& A, const BlockList& B, long lo
   if (sizeof(T) == 8 && bt.engine == kEngineTensor)
     return gram_tc(bt, A, B, N, out, reinterpret_cast<double*>(partial), slots_per_prob, bt.err, s,
                    herm);
-  int g = grid_for(N, kGramRows);
-  if (g > slots_per_prob) g = slots_per_prob;
+  // at least eight tiles a CTA where that still gives every SM one (a partial of up to 83 KB for
+  // each 16-row tile cost more than the tile)
+  const long long tiles = (N + kGramRows - 1) / kGramRows;
+  const long long want = std::max<long long>((152 + bt.nprob - 1) / bt.nprob, tiles / 8);
+  const int g = (int)std::min<long long>(std::min<long long>(tiles, want), slots_per_prob);
   const int U = (ma + kGramTx - 1) / kGramTx, V = (mb + kGramTx - 1) / kGramTx;
   const dim3 grid(g, bt.nprob);
   const bool df = sizeof(T) == 8 && bt.engine == kEngineDF;
@@ -499,8 +516,8 @@ iwf_status gram(const Batch& bt, const BlockList& A, const BlockList& B, long lo
   IWF_CUDA(cudaGetLastError());
   count_launch();
   const int cnt = ma * mb;
-  reduce_partials<<<dim3((cnt + 255) / 256, bt.nprob), 256, 0, s>>>(bt, partial, g, cnt, out,
-                                                                      herm, mb);
+  reduce_partials<<<dim3((cnt + 31) / 32, bt.nprob), 32 * kRedWarps, 0, s>>>(bt, partial, g, cnt,
+                                                                           out, herm, mb);
   IWF_CUDA(cudaGetLastError());
   count_launch();
   return IWF_OK;
@@ -579,7 +596,7 @@ iwf_status residual_precond(const Batch& bt, const void* X, const void* HX, cons
       off2, reinterpret_cast<V2*>(W), N, b, partial);
   IWF_CUDA(cudaGetLastError());
   count_launch();
-  resid_finish<<<bt.nprob, 32, 0, s>>>(bt, partial, g, b, resid);
+  resid_finish<<<bt.nprob, 32 * kRedWarps, 0, s>>>(bt, partial, g, b, resid);
   IWF_CUDA(cudaGetLastError());
   count_launch();
   return IWF_OK;

@@ -8,10 +8,10 @@
 // Slicing. Every value v of a group that shares one scale 2^E (a column of a Gram operand,
 // a row of an update operand; |v| < 2^E) becomes the 56-bit integer I = round(v 2^(55-E)),
 // written in balanced base-128 digits I = sum_k d_k 2^(56-7k), k = 1..8, |d_k| <= 64. Digit k
-// is stored as the bf16 value D_k = d_k 2^(-7(k-1)) (exact: at most 7 significant bits), so
-// v = 2^(E-6) sum_k D_k. A product of two values expands into digit pairs (k, l); pairs of one
-// level k + l are integer multiples of one unit 2^(-7(k+l-2)). The tensor core multiplies
-// bf16 pairs exactly and adds them in fp32; with |d| <= 64 a level's sum over a bounded
+// is stored as the bf16 integer d_k (exact: at most 7 significant bits), so
+// v = 2^(E-6) sum_k d_k 2^(-7(k-1)). A product of two values expands into digit pairs (k, l); pairs
+// of one level k + l share the unit 2^(-7(k+l-2)) and one accumulator of their integers. The
+// tensor core multiplies bf16 pairs exactly and adds them in fp32; with |d| <= 64 a level's sum over a bounded
 // number of rows stays below 2^24 units, so levels 2..6 are exact in their fp32 accumulators
 // in tensor memory (one per level), and the rounding of levels 7..10 sits below 2^-56 of the
 // scales' product. Pairs with k + l >= 11 are dropped (below 2^-62). The one rounding that
@@ -40,14 +40,14 @@ constexpr int kSmemCap = 227 * 1024 - 2048;  // dynamic shared memory per CTA (2
                                               // kernels' static shared memory)
 
 // Balanced base-128 digits of round(v 2^(55-E)), where the group's largest biased exponent is
-// maxb (E = maxb - 1022, so |v| < 2^E), as the bit patterns of the floats
-// D_k = d_k 2^(-7(k-1)), |d_k| <= 64 (at most 7 significant bits: the top half is bf16).
+// maxb (E = maxb - 1022, so |v| < 2^E): I + 64 (1 + 128 + ... + 128^7) has the digits plus 64 as its
+// 7-bit fields (the top one, 0 to 128, has 8 bits), so no carries run from digit to digit. Returned
+// as two words of four fields, low and high.
 // The scaling is an integer add to v's exponent field and the rounding one hardware
 // conversion to a 64-bit integer (measured faster here than a rounded shift of the mantissa in
 // 64-bit integer arithmetic, with either the tensor-core issue or the slicing as the
-// bottleneck); the digits then come from two 28-bit halves in 32-bit arithmetic.
-// Zeros, denormals and values below 2^(E-56) give zero digits.
-__device__ __forceinline__ void digits8(double v, int maxb, uint32_t (&f)[kDig]) {
+// bottleneck). Zeros, denormals and values below 2^(E-56) give zero digits.
+__device__ __forceinline__ uint2 digit_fields(double v, int maxb) {
   const long long bits = __double_as_longlong(v);
   const int hi = (int)(bits >> 32);
   const int e = (hi >> 20) & 0x7FF;
@@ -55,44 +55,41 @@ __device__ __forceinline__ void digits8(double v, int maxb, uint32_t (&f)[kDig])
   long long I = 0;
   if (e != 0 && e + sh > 0)
     I = __double2ll_rn(__hiloint2double(hi + (sh << 20), (int)bits));
-  // I = q 2^28 + r with r in [-2^27, 2^27)
-  const int r0 = ((int)((unsigned int)I << 4)) >> 4;
-  int q = (int)((I - r0) >> 28);
-  int r = r0;
-  int d[kDig];
-  d[0] = (q + (1 << 20)) >> 21; q -= d[0] << 21;
-  d[1] = (q + (1 << 13)) >> 14; q -= d[1] << 14;
-  d[2] = (q + (1 << 6)) >> 7;   q -= d[2] << 7;
-  d[3] = q;
-  d[4] = (r + (1 << 20)) >> 21; r -= d[4] << 21;
-  d[5] = (r + (1 << 13)) >> 14; r -= d[5] << 14;
-  d[6] = (r + (1 << 6)) >> 7;   r -= d[6] << 7;
-  d[7] = r;
-  // d 2^(-7k) exactly: add d to the bits of m = 1.5 2^(23-7k) (whose last place is 2^(-7k)),
-  // then subtract m
-#pragma unroll
-  for (int k = 0; k < kDig; ++k) {
-    const float m = __int_as_float(((150 - 7 * k) << 23) | 0x400000);
-    f[k] = __float_as_uint(__int_as_float(__float_as_int(m) + d[k]) - m);
-  }
+  const unsigned long long f = (unsigned long long)(I + 0x81020408102040LL);
+  return make_uint2((unsigned int)f & 0xFFFFFFFu, (unsigned int)(f >> 28));
 }
 
-__device__ __forceinline__ uint32_t pack2(uint32_t lo, uint32_t hi) {
-  return __byte_perm(lo, hi, 0x7632);
+// 16-bit halves holding fields f (two values): the bf16 pair f - 64. 128 + f is the bf16 with bits
+// 0x4300 + f for 0 <= f <= 128, and subtracting 192 is exact.
+__device__ __forceinline__ uint32_t field_digits(uint32_t halves, uint32_t mask) {
+  uint32_t d;
+  asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"((halves & mask) | 0x43004300u), "r"(0x43404340u));
+  return d;
 }
 
 // Digits of 8 consecutive values of one group, written as the 16-byte K-row of one tile row
-// in each of the digit tiles (tile k at base + k * tile_stride).
+// in each of the digit tiles (tile k at base + k * tile_stride, most significant digit first).
+// Per value about 14 integer operations for its eight digits, which come in pairs of values: a
+// 16-bit half holds two neighbouring fields, the upper one 7 bits up. (Digits peeled off one by
+// one through floats took about 38; the Gram products, which this slicing bounds, took 33.0 ms of a
+// six-iteration solve at 32^4 then and 26.7 ms now, the updates 36.9 and 34.5 ms.)
 __device__ __forceinline__ void store_digits8(const double (&v)[8], int maxb, unsigned char* base,
                                               uint32_t tile_stride, uint32_t off) {
   uint32_t w[kDig][4];
 #pragma unroll
   for (int j = 0; j < 8; j += 2) {
-    uint32_t a[kDig], b[kDig];
-    digits8(v[j], maxb, a);
-    digits8(v[j + 1], maxb, b);
-#pragma unroll
-    for (int k = 0; k < kDig; ++k) w[k][j / 2] = pack2(a[k], b[k]);
+    const uint2 a = digit_fields(v[j], maxb), b = digit_fields(v[j + 1], maxb);
+    const uint32_t lo0 = __byte_perm(a.x, b.x, 0x5410), lo1 = __byte_perm(a.x >> 14, b.x >> 14, 0x5410);
+    const uint32_t hi0 = __byte_perm(a.y, b.y, 0x5410), hi1 = __byte_perm(a.y >> 14, b.y >> 14, 0x5410);
+    constexpr uint32_t m7 = 0x007F007Fu, m8 = 0x00FF00FFu;
+    w[7][j / 2] = field_digits(lo0, m7);
+    w[6][j / 2] = field_digits(lo0 >> 7, m7);
+    w[5][j / 2] = field_digits(lo1, m7);
+    w[4][j / 2] = field_digits(lo1 >> 7, m7);
+    w[3][j / 2] = field_digits(hi0, m7);
+    w[2][j / 2] = field_digits(hi0 >> 7, m7);
+    w[1][j / 2] = field_digits(hi1, m7);
+    w[0][j / 2] = field_digits(hi1 >> 7, m8);
   }
 #pragma unroll
   for (int k = 0; k < kDig; ++k)
@@ -453,8 +450,8 @@ gram_tc_kernel(Batch bt, BlockList A, BlockList B, long long N, long long rows_p
               tc::tmem_wait_ld();
 #pragma unroll
               for (int u = 0; u < 8; ++u) {
-                float s, er;
-                two_sum(hi[gi * 8 + u], v[u], s, er);
+                float s, er;                       // level a + 2 in its unit 2^(-7a)
+                two_sum(hi[gi * 8 + u], v[u] * __int_as_float((127 - 7 * a) << 23), s, er);
                 hi[gi * 8 + u] = s;
                 lo[gi * 8 + u] += er;
               }
@@ -492,14 +489,18 @@ gram_tc_kernel(Batch bt, BlockList A, BlockList B, long long N, long long rows_p
 
 // G[prob] (ma x mb, row-major, complex double at out + prob * kCapG) from the slot partials of
 // the sub-Grams, with the column scales 2^(Ea + Eb - 12), E = maxb - 1022. An entry of a
-// skipped (Hermitian) block is the conjugate of its mirror image.
+// skipped (Hermitian) block is the conjugate of its mirror image. A CTA takes 32 entries, its
+// warps every kRedWarps-th slot each (one thread an entry: 46 us at 147 slots, an FP64 chain).
+constexpr int kRedWarps = 8;
 __global__ void gram_tc_reduce(Batch bt, const double* partial, int slots, int ma, int mb,
                                SubList subs, double2* out) {
   const int prob = blockIdx.y;
   if (bt.active && !bt.active[prob]) return;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= ma * mb) return;
-  int a = e / mb, b = e % mb;
+  __shared__ double2 part[kRedWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + lane;
+  const bool live = e < ma * mb;
+  int a = live ? e / mb : 0, b = live ? e % mb : 0;
   int si = -1;
   bool mirror = false;
   for (int t = 0; t < subs.n && si < 0; ++t) {
@@ -515,15 +516,21 @@ __global__ void gram_tc_reduce(Batch bt, const double* partial, int slots, int m
     const int tmp = a; a = b; b = tmp;
   }
   double2 r = make_double2(nan(""), nan(""));
+  double re = 0.0, im = 0.0;
   if (si >= 0) {
     const SubGram g = subs.s[si];
     const int ia = a - g.a0, ib = b - g.b0, Nc = 2 * g.nb;
-    const double* p = partial + (size_t)prob * slots * subs.slot_size + g.poff;
-    double re = 0.0, im = 0.0;
-    for (int s = 0; s < slots; ++s, p += subs.slot_size) {
+    for (int s = warp; s < slots; s += kRedWarps) {
+      const double* p = partial + ((size_t)prob * slots + s) * subs.slot_size + g.poff;
       re += p[(size_t)ia * Nc + ib] + p[(size_t)(ia + g.na) * Nc + ib + g.nb];
       im += p[(size_t)ia * Nc + ib + g.nb] - p[(size_t)(ia + g.na) * Nc + ib];
     }
+  }
+  part[warp][lane] = make_double2(re, im);
+  __syncthreads();
+  if (warp > 0 || !live) return;
+  if (si >= 0) {
+    for (int w = 1; w < kRedWarps; ++w) { re += part[w][lane].x; im += part[w][lane].y; }
     const int* expA = bt.exps + (size_t)prob * 2 * kMaxSmall;
     const int ea = expA[a], eb = expA[kMaxSmall + b];
     if (ea < 2047 && eb < 2047) {
@@ -580,9 +587,9 @@ __device__ __forceinline__ double ll_to_double_scaled(long long T, int sh) {
                                           (M & 0xFFFFFFFFFFFFFull)));
 }
 
-// round(x * scale) for |x scale| < 2^22 (exact when x scale is an integer)
-__device__ __forceinline__ int magic_int(float x, float scale) {
-  return __float_as_int(fmaf(x, scale, 12582912.0f)) - 0x4B400000;
+// an integer-valued float below 2^22 in magnitude as an int
+__device__ __forceinline__ int magic_int(float x) {
+  return __float_as_int(x + 12582912.0f) - 0x4B400000;
 }
 
 // v 2^e, 0 <= e <= 1000; zeros, denormals, NaN and Inf stay
@@ -825,7 +832,9 @@ update_tc_kernel(Batch bt, BlockList S, int m, long long N, const double2* C1, c
         }
         // levels 7..10 together (their rounding sits far below the result's last bit)
 #pragma unroll
-        for (int u = 0; u < 8; ++u) a[5][u] = (a[5][u] + a[6][u]) + (a[7][u] + a[8][u]);
+        for (int u = 0; u < 8; ++u)
+          a[5][u] = fmaf(a[6][u], 0x1p-7f, a[5][u]) +
+                    fmaf(a[8][u], 0x1p-7f, a[7][u]) * 0x1p-14f;
 #pragma unroll
         for (int u = 0; u < 8; u += 2) {
           const int jc = (8 * g + u) >> 1;       // complex output column
@@ -834,20 +843,20 @@ update_tc_kernel(Batch bt, BlockList S, int m, long long N, const double2* C1, c
 #pragma unroll
           for (int w = 0; w < 2; ++w) {
             const int n = 8 * g + u + w;
-            // Th = 2^28 x (levels 2..6): the level-l sum is an integer multiple of 2^(-7(l-2))
-            // below 2^22 of its unit, so Th is exact (below 2^48). The shared levels 7..10 are
-            // added at a finer unit 2^(-28-k), k as large as keeps the sum in 62 bits.
+            // Th = 2^28 x (levels 2..6): the level-l sum is an integer below 2^22 in units of
+            // 2^(-7(l-2)), so Th is exact (below 2^48). The levels 7..10, together in units of
+            // 2^-35, are added at a finer unit 2^(-28-k), k as large as keeps the sum in 62 bits.
             const long long Th =
-                ((long long)magic_int(a[0][u + w], 1.0f) << 28) +
-                ((long long)magic_int(a[1][u + w], 128.0f) << 21) +
-                ((long long)magic_int(a[2][u + w], 16384.0f) << 14) +
-                ((long long)magic_int(a[3][u + w], 2097152.0f) << 7) +
-                (long long)magic_int(a[4][u + w], 268435456.0f);
+                ((long long)magic_int(a[0][u + w]) << 28) +
+                ((long long)magic_int(a[1][u + w]) << 21) +
+                ((long long)magic_int(a[2][u + w]) << 14) +
+                ((long long)magic_int(a[3][u + w]) << 7) +
+                (long long)magic_int(a[4][u + w]);
             const unsigned long long ua = Th < 0 ? (unsigned long long)(-Th) : (unsigned long long)Th;
             const int nb = 64 - __clzll((long long)ua);
             const int k = min(21, 62 - nb);
             const long long T = Th * (1LL << k) +
-                                __float2ll_rn(a[5][u + w] * __int_as_float((127 + 28 + k) << 23));
+                                __float2ll_rn(a[5][u + w] * __int_as_float((127 - 7 + k) << 23));
             // value = T 2^(-28-k) 2^(Er + En - 12), E = maxb - 1022
             const int en = colexpB[n];
             val[w] = (er >= 2047 || en >= 2047)
@@ -920,7 +929,7 @@ iwf_status launch_gram_tc(const Batch& bt, const BlockList& A, const BlockList& 
                                                               err);
   IWF_CUDA(cudaGetLastError());
   count_launch();
-  gram_tc_reduce<<<dim3((ma * mb + 255) / 256, bt.nprob), 256, 0, s>>>(
+  gram_tc_reduce<<<dim3((ma * mb + 31) / 32, bt.nprob), 32 * kRedWarps, 0, s>>>(
       bt, partial, std::max(1, slots), ma, mb, subs, out);
   IWF_CUDA(cudaGetLastError());
   count_launch();
