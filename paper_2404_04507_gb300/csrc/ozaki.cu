@@ -544,14 +544,20 @@ __global__ void gram_tc_reduce(Batch bt, const double* partial, int slots, int m
 // ---------------------------------------------------------------------------------------
 // Update kernel: Y_o = S C_o (or Y_0 -= S C_0) for 128-row tiles of S. MMA M = 128 rows,
 // N = 2q (row 2j of B gives Re Y_j, row 2j+1 Im Y_j), K = 2m with the re and im parts of each
-// S column interleaved. Row scales of S come from a first pass over the tile (its data then
-// sits in L2 for the second pass that slices it); column scales of C are computed once per
-// CTA. One CTA per SM, persistent over tiles; blockIdx.x = 2 * slot + o for two outputs, so
-// that the two CTAs reading one tile run side by side. Roles: warps 0..7 slice (K16 slices of
-// 8 S columns into a 3-slot ring), warp 8 issues the MMAs, warps 9..12 assemble the FP64
-// outputs from the level accumulators with integer arithmetic.
-constexpr int kUpdProd = 8, kUpdEpi = 4;
-constexpr int kUpdThreads = (kUpdProd + 1 + kUpdEpi) * 32;
+// S column interleaved. Column scales of C are computed once per CTA. One CTA per SM, persistent
+// over tiles; blockIdx.x = 2 * slot + o for two outputs, so that the two CTAs reading one tile run
+// side by side. Roles: warps 0..7 slice (K16 slices of 8 S columns into a 3-slot ring), warp 8
+// issues the MMAs, warps 9..16 assemble the FP64 outputs from the level accumulators with integer
+// arithmetic, warps 17..20 find the row scales of the tiles ahead.
+// A tile's MMAs and the reading of its accumulators take turns (nine levels of 48 columns fill
+// tensor memory), so the assembly bounds short contractions. In us for 2^20 rows, 24 outputs:
+// m = 24 337, m = 72 667, 48 columns subtracted 712; with four assembly warps, a variable binary
+// point, old values loaded where they are needed and the slicing warps finding the scales in a
+// pass of their own 694, 1035 and 1465. Two warps for the row scales took 2117 (m = 72), tiles
+// dealt round-robin instead of in runs 769 (subtracted).
+constexpr int kUpdProd = 8, kUpdEpi = 8;
+constexpr int kUpdRow = 4;
+constexpr int kUpdThreads = (kUpdProd + 1 + kUpdEpi + kUpdRow) * 32;
 constexpr int kUpdSlots = 3;
 constexpr int kRxRing = 2;                               // row-scale buffers in flight
 constexpr int kTileA = 128 * tc::kTileRowBytes;          // 4 KB: 128 rows x K16
@@ -565,26 +571,20 @@ struct UpdCfg {
   static constexpr int kSmem = kBBytes + kUpdSlots * kUpdSliceBytes + 1024;
 };
 
-// FP64 value of T * 2^(sh) for a 64-bit integer T (round to nearest; 0 below the normal range).
+// FP64 value of T * 2^(sh) for a 64-bit integer T, |T| < 2^63 (round to nearest; 0 below the normal
+// range).
 __device__ __forceinline__ double ll_to_double_scaled(long long T, int sh) {
-  if (T == 0) return 0.0;
-  const unsigned long long sign = T < 0 ? (1ull << 63) : 0ull;
-  unsigned long long U = T < 0 ? (unsigned long long)(-T) : (unsigned long long)T;
+  const unsigned long long U = T < 0 ? 0ull - (unsigned long long)T : (unsigned long long)T;
   const int lz = __clzll((long long)U);
-  int top = 63 - lz;                       // position of the leading one
-  unsigned long long M;
-  if (top > 52) {
-    const int r = top - 52;
-    M = (U + (1ull << (r - 1))) >> r;      // may carry into bit 53
-    if (M >> 53) { M >>= 1; ++top; }
-  } else {
-    M = U << (52 - top);
-  }
-  const int e = top + sh + 1023;
-  if (e <= 0) return 0.0;
-  if (e >= 2047) return __longlong_as_double((long long)(sign | (0x7FFull << 52)));
-  return __longlong_as_double((long long)(sign | ((unsigned long long)e << 52) |
-                                          (M & 0xFFFFFFFFFFFFFull)));
+  const unsigned long long n = U << (lz & 63);           // the leading one at bit 63
+  // 53 bits, rounded; the leading one and a carry out of the fraction add to the exponent field
+  const unsigned long long M = (n >> 11) + ((n >> 10) & 1ull);
+  const int e = 63 - lz + sh + 1022;
+  const unsigned long long sign = (unsigned long long)T & (1ull << 63);
+  unsigned long long r = ((unsigned long long)e << 52) + M;
+  if (e < 0 || U == 0) r = 0;
+  if (e >= 2046) r = 0x7FFull << 52;
+  return __longlong_as_double((long long)(sign | r));
 }
 
 // an integer-valued float below 2^22 in magnitude as an int
@@ -623,6 +623,7 @@ update_tc_kernel(Batch bt, BlockList S, int m, long long N, const double2* C1, c
   double2* Y = (o == 0 ? out1 : out2) + poff;
   const int nsl = (m + 7) / 8;                  // K16 slices (8 S columns each)
   const long long ntiles = (N + 127) / 128;
+  const long long t_begin = ntiles * slot / nslots, t_end = ntiles * (slot + 1) / nslots;
   unsigned char* Bt = smem;                     // [slice][digit] B tiles
   unsigned char* ring = smem + Cfg::kBBytes;    // [slot][digit] A tiles
 
@@ -658,8 +659,8 @@ update_tc_kernel(Batch bt, BlockList S, int m, long long N, const double2* C1, c
     tc::bar_init(tc::smem_u32(&acce_bar), kUpdEpi * 32);
     tc::bar_init(tc::smem_u32(&done_bar), 1);
     for (int i = 0; i < kRxRing; ++i) {
-      tc::bar_init(tc::smem_u32(&rxf_bar[i]), kUpdProd * 32);
-      tc::bar_init(tc::smem_u32(&rxe_bar[i]), kUpdEpi * 32);
+      tc::bar_init(tc::smem_u32(&rxf_bar[i]), kUpdRow * 32);
+      tc::bar_init(tc::smem_u32(&rxe_bar[i]), (kUpdEpi + kUpdProd) * 32);
     }
     tc::bar_init_fence();
     abort_flag = 0;
@@ -701,56 +702,34 @@ update_tc_kernel(Batch bt, BlockList S, int m, long long N, const double2* C1, c
     // ---- producers: thread (rho, hh) owns row rho of the tile and half of its columns;
     // both halves of a row sit in one warp, so the row's scale is a shuffle away ----
     const int rho = warp * 16 + (lane & 15), hh = lane >> 4;
-    const auto ld = [&](int c, long long r) { return scol[c][r]; };
     int j = 0;                                  // slices produced so far (ring position)
     int tcount = 0;
-    for (long long t = slot; t < ntiles && !*abort_v; t += nslots, ++tcount) {
+    for (long long t = t_begin; t < t_end && !*abort_v; ++t, ++tcount) {
       const long long r = t * 128 + rho;
       const bool live = r < N;
-      // pass 1: this row's largest exponent over all of S's columns, eight loads in flight
-      unsigned int mx = 0;
-      if (live) {
-        for (int c0 = hh; c0 < m; c0 += 16) {
-          double2 v[8];
+      // slices of 8 columns (this thread: 4 columns, re and im, of its row); the values of the next
+      // two slices are loaded before this one is sliced
+      const auto fetch = [&](int sl, double2 (&o)[4]) {
 #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int c = c0 + 2 * u;
-            v[u] = c < m ? ld(c, r) : make_double2(0.0, 0.0);
-          }
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const unsigned int hx = (unsigned int)(__double_as_longlong(v[u].x) >> 32);
-            const unsigned int hy = (unsigned int)(__double_as_longlong(v[u].y) >> 32);
-            mx = max(mx, max((hx >> 20) & 0x7FFu, (hy >> 20) & 0x7FFu));
-          }
+        for (int u = 0; u < 4; ++u) {
+          const int c = 8 * sl + 4 * hh + u;
+          o[u] = (live && c < m) ? scol[c][r] : make_double2(0.0, 0.0);
         }
-      }
-      mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
-      const int maxb = (int)mx;
-      // the row scales travel to the epilogue through a ring of buffers
+      };
+      double2 cur[4], nxt[4], far[4];
+      fetch(0, cur);
+      fetch(1, nxt);
       const int rb = tcount % kRxRing;
-      if (!wait_bounded(tc::smem_u32(&rxe_bar[rb]), (uint32_t)(((tcount / kRxRing) & 1) ^ 1))) {
+      if (!wait_bounded(tc::smem_u32(&rxf_bar[rb]), (uint32_t)((tcount / kRxRing) & 1))) {
         atomicExch(&abort_flag, 1);
         break;
       }
-      if (hh == 0) rowexp[rb][rho] = maxb;
-      tc::bar_arrive(tc::smem_u32(&rxf_bar[rb]));
-      // pass 2: slices of 8 columns (this thread: 4 columns, re and im, of its row); the next
-      // slice's values are loaded before this one is sliced
-      double2 cur[4], nxt[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int c = 4 * hh + u;
-        cur[u] = (live && c < m) ? ld(c, r) : make_double2(0.0, 0.0);
-      }
+      const int maxb = rowexp[rb][rho];
+      tc::bar_arrive(tc::smem_u32(&rxe_bar[rb]));
       bool ok = true;
       for (int sl = 0; sl < nsl; ++sl, ++j) {
         const int st = j % kUpdSlots;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int c = 8 * (sl + 1) + 4 * hh + u;
-          nxt[u] = (live && c < m) ? ld(c, r) : make_double2(0.0, 0.0);
-        }
+        fetch(sl + 2, far);
         if (!wait_bounded(tc::smem_u32(&empty_bar[st]), (uint32_t)(((j / kUpdSlots) & 1) ^ 1))) {
           atomicExch(&abort_flag, 1);
           ok = false;
@@ -763,7 +742,7 @@ update_tc_kernel(Batch bt, BlockList S, int m, long long N, const double2* C1, c
         tc::fence_async_smem();
         tc::bar_arrive(tc::smem_u32(&full_bar[st]));
 #pragma unroll
-        for (int u = 0; u < 4; ++u) cur[u] = nxt[u];
+        for (int u = 0; u < 4; ++u) { cur[u] = nxt[u]; nxt[u] = far[u]; }
       }
       if (!ok) break;
     }
@@ -772,7 +751,7 @@ update_tc_kernel(Batch bt, BlockList S, int m, long long N, const double2* C1, c
     if (lane == 0) {
       const uint32_t idn = tc::idesc_bf16(128, NMMA, false);
       int j = 0, tcount = 0;
-      for (long long t = slot; t < ntiles && !*abort_v; t += nslots, ++tcount) {
+      for (long long t = t_begin; t < t_end && !*abort_v; ++t, ++tcount) {
         if (tcount > 0 &&
             !wait_bounded(tc::smem_u32(&acce_bar), (uint32_t)((tcount - 1) & 1))) {
           atomicExch(&abort_flag, 1);
@@ -800,18 +779,59 @@ update_tc_kernel(Batch bt, BlockList S, int m, long long N, const double2* C1, c
       wait_bounded(tc::smem_u32(&done_bar), 0);
     }
     __syncwarp();
+  } else if (warp > kUpdProd + kUpdEpi) {
+    // ---- row scales, up to kRxRing tiles ahead of the slices: the largest exponent of each row
+    // over all of S's columns (which also brings the tile into L2 for the slicing warps) ----
+    const int rho = threadIdx.x - (kUpdProd + 1 + kUpdEpi) * 32;
+    int tcount = 0;
+    for (long long t = t_begin; t < t_end && !*abort_v; ++t, ++tcount) {
+      const long long r = t * 128 + rho;
+      unsigned int mx = 0;
+      for (int c0 = 0; r < N && c0 < m; c0 += 12) {
+        double2 v[12];
+#pragma unroll
+        for (int u = 0; u < 12; ++u)
+          v[u] = c0 + u < m ? scol[c0 + u][r] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int u = 0; u < 12; ++u) {
+          const unsigned int hx = (unsigned int)__double2hiint(v[u].x);
+          const unsigned int hy = (unsigned int)__double2hiint(v[u].y);
+          mx = max(mx, max((hx >> 20) & 0x7FFu, (hy >> 20) & 0x7FFu));
+        }
+      }
+      const int rb = tcount % kRxRing;
+      if (!wait_bounded_sleep(tc::smem_u32(&rxe_bar[rb]), (uint32_t)(((tcount / kRxRing) & 1) ^ 1))) {
+        atomicExch(&abort_flag, 1);
+        break;
+      }
+      rowexp[rb][rho] = (int)mx;
+      tc::bar_arrive(tc::smem_u32(&rxf_bar[rb]));
+    }
   } else {
     // ---- epilogue: lanes are rows; FP64 assembly with integer arithmetic ----
     const int qd = warp & 3;
     const int rho = 32 * qd + lane;
+    constexpr int G = NMMA / 8;                   // groups of four complex columns, two halves
+    const int half = (warp - kUpdProd - 1) >> 2;
+    const int g0 = half ? (G + 1) / 2 : 0, g1 = half ? G : (G + 1) / 2;
+    static_assert(G >= 2, "both halves have a group");
     int tcount = 0;
-    for (long long t = slot; t < ntiles && !*abort_v; t += nslots, ++tcount) {
+    for (long long t = t_begin; t < t_end && !*abort_v; ++t, ++tcount) {
+      const long long r = t * 128 + rho;
+      // SUB: the values to subtract from, loaded a group of four columns ahead of their use (the
+      // first group's before the wait)
+      double2 old[4], next[4];
+      const auto prefetch = [&](int g, double2 (&o)[4]) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (4 * g + u < q && r < N) o[u] = Y[(size_t)(4 * g + u) * N + r];
+      };
+      if (SUB && g0 < g1) prefetch(g0, old);
       if (!wait_bounded_sleep(tc::smem_u32(&accf_bar), (uint32_t)(tcount & 1))) {
         atomicExch(&abort_flag, 1);
         break;
       }
       tc::fence_after_sync();
-      const long long r = t * 128 + rho;
       const int rb = tcount % kRxRing;
       if (!wait_bounded(tc::smem_u32(&rxf_bar[rb]), (uint32_t)((tcount / kRxRing) & 1))) {
         atomicExch(&abort_flag, 1);
@@ -819,14 +839,14 @@ update_tc_kernel(Batch bt, BlockList S, int m, long long N, const double2* C1, c
       }
       const int er = rowexp[rb][rho];
       tc::bar_arrive(tc::smem_u32(&rxe_bar[rb]));
-      constexpr int G = NMMA / 8;
-      for (int g = 0; g < G; ++g) {
+      for (int g = g0; g < g1; ++g) {
+        if (SUB && g + 1 < g1) prefetch(g + 1, next);
         float a[kNumLvl][8];
 #pragma unroll
         for (int ac = 0; ac < kNumLvl; ++ac)
           tc::tmem_ld8(tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(ac * NMMA + 8 * g), a[ac]);
         tc::tmem_wait_ld();
-        if (g == G - 1) {
+        if (g == g1 - 1) {
           tc::fence_before_sync();
           tc::bar_arrive(tc::smem_u32(&acce_bar));
         }
@@ -843,34 +863,31 @@ update_tc_kernel(Batch bt, BlockList S, int m, long long N, const double2* C1, c
 #pragma unroll
           for (int w = 0; w < 2; ++w) {
             const int n = 8 * g + u + w;
-            // Th = 2^28 x (levels 2..6): the level-l sum is an integer below 2^22 in units of
-            // 2^(-7(l-2)), so Th is exact (below 2^48). The levels 7..10, together in units of
-            // 2^-35, are added at a finer unit 2^(-28-k), k as large as keeps the sum in 62 bits.
-            const long long Th =
-                ((long long)magic_int(a[0][u + w]) << 28) +
-                ((long long)magic_int(a[1][u + w]) << 21) +
-                ((long long)magic_int(a[2][u + w]) << 14) +
-                ((long long)magic_int(a[3][u + w]) << 7) +
-                (long long)magic_int(a[4][u + w]);
-            const unsigned long long ua = Th < 0 ? (unsigned long long)(-Th) : (unsigned long long)Th;
-            const int nb = 64 - __clzll((long long)ua);
-            const int k = min(21, 62 - nb);
-            const long long T = Th * (1LL << k) +
-                                __float2ll_rn(a[5][u + w] * __int_as_float((127 - 7 + k) << 23));
-            // value = T 2^(-28-k) 2^(Er + En - 12), E = maxb - 1022
+            // x 2^42 = the level sums: levels 2..6 are integers below 2^22 in units of
+            // 2^(-7(l-2)), gathered exactly (below 2^62), two of them in 32 bits first; levels
+            // 7..10, together in units of 2^-35, are rounded to 2^-42 (the pairs that are dropped
+            // leave about 2^-48 of a level-2 unit)
+            const int m12 = magic_int(a[1][u + w]) * 128 + magic_int(a[2][u + w]);
+            const int m34 = magic_int(a[3][u + w]) * 128 + magic_int(a[4][u + w]);
+            const long long top = (long long)magic_int(a[0][u + w]) * 16384 + m12;
+            const long long T = (((top << 14) + m34) << 14) + __float2int_rn(a[5][u + w] * 128.0f);
+            // value = T 2^-42 2^(Er + En - 12), E = maxb - 1022
             const int en = colexpB[n];
             val[w] = (er >= 2047 || en >= 2047)
                          ? nan("")
-                         : ll_to_double_scaled(T, er + en - 2044 - 12 - 28 - k);
+                         : ll_to_double_scaled(T, er + en - 2044 - 12 - 42);
           }
           double2* dst = Y + (size_t)jc * N + r;
           if (SUB) {
-            const double2 old = *dst;
-            *dst = make_double2(scale_up(old.x - val[0], col_up[jc]),
-                                scale_up(old.y - val[1], col_up[jc]));
+            *dst = make_double2(scale_up(old[u / 2].x - val[0], col_up[jc]),
+                                scale_up(old[u / 2].y - val[1], col_up[jc]));
           } else {
             *dst = make_double2(val[0], val[1]);
           }
+        }
+        if (SUB) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) old[u] = next[u];
         }
       }
     }
