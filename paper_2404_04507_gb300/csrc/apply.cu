@@ -24,6 +24,7 @@
 // k_II axes of equal lengths 16 or 32 (the 2D moire family): one pencil per thread in
 // registers, global loads and stores straight from registers, one swizzled shared-memory
 // transpose per axis change, and for complex float a bulk-copy pipeline in pass C.
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 #include <string>
@@ -945,9 +946,18 @@ int long_group_values(const PassArgs& a) {
   return v;
 }
 
-// Choose C (inner chunk) and Ot (outer indices) for a group pass within tile_kb of smem.
+// Warps that run the DFTs of `outer` outer indices of a tile along every axis of a codelet group
+// (one thread a pencil), over the axes.
+long long tile_warps(const PassArgs& a, long long outer) {
+  long long w = 0;
+  for (int ax = 0; ax < a.grp.ng; ++ax) w += (outer * (a.M / a.grp.len[ax]) * a.C + 31) / 32;
+  return w;
+}
+
+// Choose C (inner chunk) and Ot (outer indices) for a group pass within tile_kb of smem; nv:
+// vectors of a launch.
 template <typename T>
-void choose_tile(PassArgs& a, int tile_kb) {
+void choose_tile(PassArgs& a, int tile_kb, int nv) {
   // pass B (inner > 1) also keeps its group's V table (M values) next to the tile
   long long kb = (long long)tile_kb * 1024 - (a.inner > 1 ? (long long)a.M * sizeof(T) : 0);
   if (kb < 0) kb = 0;
@@ -961,8 +971,27 @@ void choose_tile(PassArgs& a, int tile_kb) {
     ot = ot < 1 ? 1 : ot;
     // keep several tiles per SM worth of parallelism
     const long long want = (a.outer + 4 * 152 - 1) / (4 * 152);
-    if (ot > want) ot = want < 1 ? 1 : want;
-    if (ot > 64) ot = 64;
+    if (vmin > 0) {
+      if (ot > want) ot = want < 1 ? 1 : want;
+      if (ot > 64) ot = 64;
+    } else {
+      // a codelet runs on one thread a pencil, and a slice may have few (18 at 18 x 18): as many
+      // slices as fill whole warps (within 5 % of the fewest warps a slice), up to 256 pencils, over
+      // all vectors of the launch still three tiles an SM. An FP64 instruction costs a warp the
+      // same with 18 lanes as with 32. Transforms in complex double, us, one slice a tile (in
+      // CTAs of 256 threads) before: 18^2 x 22^2, 6 vectors 1027 -> 353; 22^4, 24 vectors 5580 ->
+      // 2223; 10^4, 24 vectors 378 -> 88; slices of 12^3, which fill CTAs alone, as before.
+      const long long most = std::min<long long>(std::min<long long>(ot, 64), a.outer);
+      ot = 1;
+      double best = (double)tile_warps(a, 1);
+      int shortest = a.grp.len[0];
+      for (int ax = 1; ax < a.grp.ng; ++ax) shortest = std::min(shortest, a.grp.len[ax]);
+      for (long long o = 2; o <= most && o * (a.M / shortest) <= kThreads; ++o) {
+        if ((a.outer + o - 1) / o * nv < 3 * 152) break;
+        const double cost = (double)tile_warps(a, o) / (double)o;
+        if (cost < 0.95 * best) { best = cost; ot = o; }
+      }
+    }
     a.Ot = (int)ot;
   } else {
     a.Ot = 1;
@@ -1011,7 +1040,16 @@ iwf_status launch_pass(PassArgs a, int nvec, cudaStream_t stream, PassTimer* tim
   IWF_TRY((pass_smem<T, KIND>(a, &tbytes, &bytes)));
   a.tile_bytes = (int)tbytes;
   const int vmin = long_group_values(a);
-  if (vmin > 0) threads = kLongThreads;
+  if (vmin > 0) {
+    threads = kLongThreads;
+  } else {
+    // no more threads than the tile has pencils (one thread runs one): the rest would only hold
+    // registers that other CTAs of the SM need
+    int most = 1;
+    for (int ax = 0; ax < a.grp.ng; ++ax) most = std::max(most, a.Ot * (a.M / a.grp.len[ax]) * a.C);
+    const int rounds = (most + threads - 1) / threads;
+    threads = std::min(threads, std::max(64, ((most + rounds - 1) / rounds + 31) / 32 * 32));
+  }
   static bool attr_set[2][4][2] = {};
   const int ti = sizeof(T) == 8 ? 0 : 1;
   const int li = vmin > 0 ? 1 : 0;
@@ -1244,7 +1282,7 @@ iwf_status apply_typed(iwf_plan* p, const void* psi, void* hpsi, int nvec, cudaS
   }
   for (int j = 0; j < d; ++j)
     A.ltw[j] = sizeof(T) == 8 ? (const void*)p->d_ltw64[j] : (const void*)p->d_ltw32[j];
-  choose_tile<T>(A, tile_kb);
+  choose_tile<T>(A, tile_kb, chunk);
 
   PassArgs B{};
   B.g = g; B.lo = p->d_lo; B.ld = g.N; B.pot = pot;
@@ -1276,10 +1314,10 @@ iwf_status apply_typed(iwf_plan* p, const void* psi, void* hpsi, int nvec, cudaS
       q.inner = g.MII / outer / g.lens[d + j] * g.MI;
       q.ii0 = j;
       outer *= g.lens[d + j];
-      choose_tile<T>(q, tile_kb);
+      choose_tile<T>(q, tile_kb, chunk);
     }
   } else {
-    choose_tile<T>(B, tile_kb);
+    choose_tile<T>(B, tile_kb, chunk);
   }
 
   // potentials with few modes need no transform; the geometries the passes refuse stay refused
