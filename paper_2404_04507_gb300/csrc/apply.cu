@@ -971,22 +971,19 @@ void choose_tile(PassArgs& a, int tile_kb, int nv) {
     ot = ot < 1 ? 1 : ot;
     // keep several tiles per SM worth of parallelism
     const long long want = (a.outer + 4 * 152 - 1) / (4 * 152);
-    if (vmin > 0) {
-      if (ot > want) ot = want < 1 ? 1 : want;
-      if (ot > 64) ot = 64;
-    } else {
+    const long long most = std::min<long long>(std::min<long long>(ot, 64), a.outer);
+    ot = std::max<long long>(1, std::min(most, want));
+    if (vmin == 0) {
       // a codelet runs on one thread a pencil, and a slice may have few (18 at 18 x 18): as many
       // slices as fill whole warps (within 5 % of the fewest warps a slice), up to 256 pencils, over
       // all vectors of the launch still three tiles an SM. An FP64 instruction costs a warp the
       // same with 18 lanes as with 32. Transforms in complex double, us, one slice a tile (in
       // CTAs of 256 threads) before: 18^2 x 22^2, 6 vectors 1027 -> 353; 22^4, 24 vectors 5580 ->
       // 2223; 10^4, 24 vectors 378 -> 88; slices of 12^3, which fill CTAs alone, as before.
-      const long long most = std::min<long long>(std::min<long long>(ot, 64), a.outer);
-      ot = 1;
-      double best = (double)tile_warps(a, 1);
+      double best = (double)tile_warps(a, ot) / (double)ot;
       int shortest = a.grp.len[0];
       for (int ax = 1; ax < a.grp.ng; ++ax) shortest = std::min(shortest, a.grp.len[ax]);
-      for (long long o = 2; o <= most && o * (a.M / shortest) <= kThreads; ++o) {
+      for (long long o = ot + 1; o <= most && o * (a.M / shortest) <= kThreads; ++o) {
         if ((a.outer + o - 1) / o * nv < 3 * 152) break;
         const double cost = (double)tile_warps(a, o) / (double)o;
         if (cost < 0.95 * best) { best = cost; ot = o; }
@@ -1047,8 +1044,7 @@ iwf_status launch_pass(PassArgs a, int nvec, cudaStream_t stream, PassTimer* tim
     // registers that other CTAs of the SM need
     int most = 1;
     for (int ax = 0; ax < a.grp.ng; ++ax) most = std::max(most, a.Ot * (a.M / a.grp.len[ax]) * a.C);
-    const int rounds = (most + threads - 1) / threads;
-    threads = std::min(threads, std::max(64, ((most + rounds - 1) / rounds + 31) / 32 * 32));
+    threads = std::min(threads, std::max(64, (most + 31) / 32 * 32));
   }
   static bool attr_set[2][4][2] = {};
   const int ti = sizeof(T) == 8 ? 0 : 1;
