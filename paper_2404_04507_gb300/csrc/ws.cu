@@ -232,7 +232,7 @@ __device__ __forceinline__ float gelu_grad_f(float z) {
 }
 
 // z = c + b (kept for the backward pass); next layer input = bf16(gelu(z)), or for the
-// output layer out = z.
+// output layer out = z (out may be null: the caller reads z).
 __global__ void bias_act(const float* c, const float* b, float* z, __nv_bfloat16* hnext,
                          float* out, int B, int N, int last) {
   const long long n = (long long)B * N;
@@ -240,7 +240,7 @@ __global__ void bias_act(const float* c, const float* b, float* z, __nv_bfloat16
        i += (long long)gridDim.x * blockDim.x) {
     const float v = c[i] + b[i % N];
     z[i] = v;
-    if (last) out[i] = v;
+    if (last) { if (out) out[i] = v; }
     else hnext[i] = __float2bfloat16_rn(gelu_f(v));
   }
 }
@@ -252,48 +252,70 @@ __global__ void act_back(const float* dh, const float* z, float* dz, long long n
     dz[i] = dh[i] * gelu_grad_f(z[i]);
 }
 
-// db[j] = sum over rows of dz[r][j]
-__global__ void colsum(const float* dz, float* db, int B, int N) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= N) return;
+// db[j] = sum over rows of dz[r][j]: a CTA takes 32 columns, its 8 warps every eighth row each
+// (one thread a column walked 256 rows one load after another: 8 us a layer).
+__global__ void __launch_bounds__(256) colsum(const float* dz, float* db, int B, int N) {
+  __shared__ float part[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int j = blockIdx.x * 32 + lane;
   float s = 0.f;
-  for (int r = 0; r < B; ++r) s += dz[(size_t)r * N + j];
+  if (j < N)
+    for (int r = warp; r < B; r += 8) s += dz[(size_t)r * N + j];
+  part[warp][lane] = s;
+  __syncthreads();
+  if (warp > 0 || j >= N) return;
+  for (int w = 1; w < 8; ++w) s += part[w][lane];
   db[j] = s;
 }
 
 // Subspace loss per sample (one CTA): Gram matrices X^H X, X^H Y, Y^H Y (nvec <= 16), then
 // dY = (-4 X (X^H Y) + 4 Y (Y^H Y)) / (B nvec) and the sample's loss / (B nvec).
+// Thread (a, c) sums its three Gram entries over chunks of core points staged in shared memory;
+// every thread adds its share of the loss. With the points read from global memory one after
+// another and the loss summed by one thread in FP64, 256 samples of 16 x 256 took 290 us.
+constexpr int kLossChunk = 64;
 __global__ void subspace_loss_kernel(const float* Y, const float* X, int nvec, int ncore,
                                      int nout, float scale, float* dY, float* loss) {
-  __shared__ float2 gxx[16][16], gxy[16][16], gyy[16][16];
+  __shared__ float2 gxy[16][16], gyy[16][16];
+  __shared__ float2 sx[16][kLossChunk + 1], sy[16][kLossChunk + 1];
+  __shared__ double red[8];
   const int s = blockIdx.x;
   const float* y = Y + (size_t)s * nout;
   const float* x = X + (size_t)s * nout;
   const int a = threadIdx.x / 16, c = threadIdx.x % 16;
-  if (a < nvec && c < nvec) {
-    float xx_r = 0, xx_i = 0, xy_r = 0, xy_i = 0, yy_r = 0, yy_i = 0;
-    for (int i = 0; i < ncore; ++i) {
-      const float2 xa = *reinterpret_cast<const float2*>(&x[((size_t)a * ncore + i) * 2]);
-      const float2 xc = *reinterpret_cast<const float2*>(&x[((size_t)c * ncore + i) * 2]);
-      const float2 ya = *reinterpret_cast<const float2*>(&y[((size_t)a * ncore + i) * 2]);
-      const float2 yc = *reinterpret_cast<const float2*>(&y[((size_t)c * ncore + i) * 2]);
+  const bool live = a < nvec && c < nvec;
+  float xx_r = 0, xx_i = 0, xy_r = 0, xy_i = 0, yy_r = 0, yy_i = 0;
+  for (int i0 = 0; i0 < ncore; i0 += kLossChunk) {
+    const int n = min(kLossChunk, ncore - i0);
+    __syncthreads();
+    for (int e = threadIdx.x; e < nvec * kLossChunk; e += blockDim.x) {
+      const int v = e / kLossChunk, i = e % kLossChunk;
+      if (i >= n) continue;
+      sx[v][i] = *reinterpret_cast<const float2*>(&x[((size_t)v * ncore + i0 + i) * 2]);
+      sy[v][i] = *reinterpret_cast<const float2*>(&y[((size_t)v * ncore + i0 + i) * 2]);
+    }
+    __syncthreads();
+    for (int i = 0; live && i < n; ++i) {
+      const float2 xa = sx[a][i], xc = sx[c][i], ya = sy[a][i], yc = sy[c][i];
       xx_r += xa.x * xc.x + xa.y * xc.y; xx_i += xa.x * xc.y - xa.y * xc.x;
       xy_r += xa.x * yc.x + xa.y * yc.y; xy_i += xa.x * yc.y - xa.y * yc.x;
       yy_r += ya.x * yc.x + ya.y * yc.y; yy_i += ya.x * yc.y - ya.y * yc.x;
     }
-    gxx[a][c] = make_float2(xx_r, xx_i);
+  }
+  double l = 0.0;
+  if (live) {
+    l = (double)xx_r * xx_r + (double)xx_i * xx_i;
+    l -= 2.0 * ((double)xy_r * xy_r + (double)xy_i * xy_i);
+    l += (double)yy_r * yy_r + (double)yy_i * yy_i;
     gxy[a][c] = make_float2(xy_r, xy_i);
     gyy[a][c] = make_float2(yy_r, yy_i);
   }
+  for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = l;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double l = 0;
-    for (int i = 0; i < nvec; ++i)
-      for (int j = 0; j < nvec; ++j) {
-        l += (double)gxx[i][j].x * gxx[i][j].x + (double)gxx[i][j].y * gxx[i][j].y;
-        l -= 2.0 * ((double)gxy[i][j].x * gxy[i][j].x + (double)gxy[i][j].y * gxy[i][j].y);
-        l += (double)gyy[i][j].x * gyy[i][j].x + (double)gyy[i][j].y * gyy[i][j].y;
-      }
+    l = 0.0;
+    for (int w = 0; w < 8; ++w) l += red[w];
     loss[s] = (float)(l * scale);
   }
   // dY[i][v] = scale * (-4 sum_a x[i][a] gxy[a][v] + 4 sum_a y[i][a] gyy[a][v])
@@ -515,13 +537,14 @@ iwf_status forward(iwf_ws* w, int B, const float* feat, float* out, cudaStream_t
   return IWF_OK;
 }
 
-// Loss and parameter gradients (into w->grads) for B samples; targets device (B x nout).
+// Loss and parameter gradients (into w->grads) for B samples; targets device (B x nout). The
+// prediction stays in the last layer's z.
 iwf_status loss_grad(iwf_ws* w, int B, const float* feat, const float* target, int nvec,
-                     int ncore, float* yout, float* loss_dev, cudaStream_t s) {
+                     int ncore, float* loss_dev, cudaStream_t s) {
   const int nout = w->dims[w->nl];
   if (2 * nvec * ncore != nout || nvec > 16) return fail(IWF_ERR_ARG, "warm start: output size != 2*nvec*ncore");
-  IWF_TRY(forward(w, B, feat, yout, s));
-  subspace_loss_kernel<<<B, 256, 0, s>>>(yout, target, nvec, ncore, nout, 1.f / (B * nvec),
+  IWF_TRY(forward(w, B, feat, nullptr, s));
+  subspace_loss_kernel<<<B, 256, 0, s>>>(w->z[w->nl - 1], target, nvec, ncore, nout, 1.f / (B * nvec),
                                          w->dz, loss_dev);
   IWF_CUDA(cudaGetLastError());
   count_launch();
@@ -533,7 +556,7 @@ iwf_status loss_grad(iwf_ws* w, int B, const float* feat, const float* target, i
     IWF_TRY(transpose(w->dzbf, w->dzt, B, o, s));
     IWF_TRY(transpose(w->hbf[l], w->ht, B, in, s));
     IWF_TRY(gemm(w, w->dzt, w->ht, w->grads + w->woff[l], o, in, B, s));
-    colsum<<<(o + 255) / 256, 256, 0, s>>>(w->dz, w->grads + w->boff[l], B, o);
+    colsum<<<(o + 31) / 32, 256, 0, s>>>(w->dz, w->grads + w->boff[l], B, o);
     count_launch();
     if (l > 0) {
       // dh = dz W  (B x in) = dz . (W^T)^T ; then dz_{l-1} = dh * gelu'(z_{l-1})
@@ -658,10 +681,8 @@ iwf_status iwf_ws_loss_grad(iwf_ws* w, int nsamples, const float* feat, const fl
     return fail(IWF_ERR_ARG, "iwf_ws_loss_grad: bad arguments (nsamples a positive multiple of 64)");
   DeviceGuard guard(w->device);
   cudaStream_t s = (cudaStream_t)stream;
-  float* y = nullptr;
-  IWF_TRY(dalloc(&y, (size_t)nsamples * w->dims[w->nl]));
   IWF_TRY(ensure_batch(w, nsamples));
-  iwf_status st = loss_grad(w, nsamples, feat, target, nvec, ncore, y, w->lossbuf, s);
+  iwf_status st = loss_grad(w, nsamples, feat, target, nvec, ncore, w->lossbuf, s);
   if (st == IWF_OK) {
     std::vector<float> l(nsamples);
     cudaMemcpyAsync(l.data(), w->lossbuf, nsamples * sizeof(float), cudaMemcpyDeviceToHost, s);
@@ -672,7 +693,6 @@ iwf_status iwf_ws_loss_grad(iwf_ws* w, int nsamples, const float* feat, const fl
     if (loss) *loss = (float)t;
     if (st == IWF_OK) st = check_ws_err(w, s);
   }
-  cudaFree(y);
   return st;
 }
 
@@ -686,14 +706,13 @@ iwf_status iwf_ws_train(iwf_ws* w, int nsamples, const float* feat, const float*
   cudaStream_t s = (cudaStream_t)stream;
   const int nin = w->dims[0], nout = w->dims[w->nl];
   IWF_TRY(ensure_batch(w, batch));
-  float *bf = nullptr, *bt = nullptr, *y = nullptr, *losses = nullptr;
+  float *bf = nullptr, *bt = nullptr, *losses = nullptr;
   int* idx = nullptr;
   unsigned char* isw = nullptr;
   const int nb = nsamples / batch;
   iwf_status st = IWF_OK;
   if (st == IWF_OK) st = dalloc(&bf, (size_t)batch * nin);
   if (st == IWF_OK) st = dalloc(&bt, (size_t)batch * nout);
-  if (st == IWF_OK) st = dalloc(&y, (size_t)batch * nout);
   if (st == IWF_OK) st = dalloc(&idx, (size_t)batch);
   if (st == IWF_OK) st = dalloc(&losses, (size_t)nb * batch);
   if (st == IWF_OK) st = dalloc(&isw, (size_t)w->nparams);
@@ -717,7 +736,7 @@ iwf_status iwf_ws_train(iwf_ws* w, int nsamples, const float* feat, const float*
       gather_rows<<<blocks_for((long long)batch * nin), 256, 0, s>>>(feat, idx, bf, batch, nin);
       gather_rows<<<blocks_for((long long)batch * nout), 256, 0, s>>>(target, idx, bt, batch, nout);
       count_launch(); count_launch();
-      st = loss_grad(w, batch, bf, bt, nvec, ncore, y, losses + (size_t)k * batch, s);
+      st = loss_grad(w, batch, bf, bt, nvec, ncore, losses + (size_t)k * batch, s);
       if (st != IWF_OK) break;
       ++w->step;
       const float c1 = 1.f - std::pow(b1, (float)w->step), c2 = 1.f - std::pow(b2, (float)w->step);
@@ -737,7 +756,7 @@ iwf_status iwf_ws_train(iwf_ws* w, int nsamples, const float* feat, const float*
       loss_hist[ep] = (float)(t / nb);
     }
   }
-  cudaFree(bf); cudaFree(bt); cudaFree(y); cudaFree(idx); cudaFree(losses); cudaFree(isw);
+  cudaFree(bf); cudaFree(bt); cudaFree(idx); cudaFree(losses); cudaFree(isw);
   return st;
 }
 
