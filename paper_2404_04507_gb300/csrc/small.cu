@@ -10,9 +10,9 @@
 //     chains that do not depend on one another on different quarters of the SM;
 //   - bisection, which needs no last bit, counts eigenvalues in double-float arithmetic on the
 //     FP32 pipes (5x the FP64 rate); inverse iteration and Rayleigh quotients are FP64.
-// Measured on one GB300, Rayleigh-Ritz with 72 basis vectors and 24 pairs: 1.25 ms (reduction 0.50,
-// bisection 0.06, inverse iteration 0.11, back-transformation and P coefficients 0.56), m = 12
-// with 4 pairs 0.14 ms. Cyclic Jacobi in double-float arithmetic, which this replaced, took 6.2
+// Measured on one GB300, Rayleigh-Ritz with 72 basis vectors and 24 pairs: 1.14 ms (reduction 0.50,
+// bisection 0.06, inverse iteration 0.11, back-transformation 0.24, P coefficients 0.23), m = 12
+// with 4 pairs 0.10 ms. Cyclic Jacobi in double-float arithmetic, which this replaced, took 6.2
 // and 0.30 ms (8 to 13 sweeps of 71 rounds at about 19k cycles) and left residuals near 1e-10 on
 // matrices with entries near 10^3; errors are now those of FP64 (residuals 2e-16 |A|).
 #include <algorithm>
@@ -517,7 +517,9 @@ __device__ void herm_eig(SmallShared& sh, int n, int k) {
     q += __shfl_xor_sync(0xffffffffu, q, 8);
     q += __shfl_xor_sync(0xffffffffu, q, 16);
     if (live && part == 0) sh.w[j] = q / scale;
-    constexpr int kPer = kMaxSmall / 4;                // rows part, part + 4, ... of the vector
+    // rows part, part + 4, ... of the vector in registers, three at a time behind a branch that the
+    // whole warp takes: an FP64 instruction that is only predicated off still costs its 64 cycles
+    constexpr int kPer = kMaxSmall / 4, kStep = 3;
     double2 y[kPer];
 #pragma unroll
     for (int t = 0; t < kPer; ++t) {
@@ -530,11 +532,16 @@ __device__ void herm_eig(SmallShared& sh, int n, int k) {
       if (tau == 0.0) continue;
       const double2* a = sh.A + c0;
       double2 s = make_double2(0.0, 0.0);
+      const auto entry = [&](int i) {                  // 0 outside the reflector
+        const double2 v = a[min(i, n - 1) * n];
+        const bool in = i > c0 && i < n;
+        return make_double2(in ? v.x : 0.0, in ? v.y : 0.0);
+      };
 #pragma unroll
-      for (int t = 0; t < kPer; ++t)
-        if (4 * t + 3 > c0 && 4 * t < n) {             // some lane's row lies below the diagonal
-          const int i = part + 4 * t;
-          if (i > c0 && i < n) s = cmac_conj(a[i * n], y[t], s);
+      for (int t0 = 0; t0 < kPer; t0 += kStep)
+        if (4 * (t0 + kStep) > c0 + 1 && 4 * t0 < n) {
+#pragma unroll
+          for (int t = t0; t < t0 + kStep; ++t) s = cmac_conj(entry(part + 4 * t), y[t], s);
         }
       s.x += __shfl_xor_sync(0xffffffffu, s.x, 8);
       s.y += __shfl_xor_sync(0xffffffffu, s.y, 8);
@@ -542,10 +549,10 @@ __device__ void herm_eig(SmallShared& sh, int n, int k) {
       s.y += __shfl_xor_sync(0xffffffffu, s.y, 16);
       s = make_double2(-tau * s.x, -tau * s.y);
 #pragma unroll
-      for (int t = 0; t < kPer; ++t)
-        if (4 * t + 3 > c0 && 4 * t < n) {
-          const int i = part + 4 * t;
-          if (i > c0 && i < n) y[t] = cmac(a[i * n], s, y[t]);
+      for (int t0 = 0; t0 < kPer; t0 += kStep)
+        if (4 * (t0 + kStep) > c0 + 1 && 4 * t0 < n) {
+#pragma unroll
+          for (int t = t0; t < t0 + kStep; ++t) y[t] = cmac(entry(part + 4 * t), s, y[t]);
         }
     }
 #pragma unroll
@@ -868,10 +875,16 @@ rr_kernel(Batch bt, const double2* Ain, int m, int b, const int* mask, int x_row
   Cp += (size_t)prob * kCapC;
   mask_p += (size_t)prob * kMaxBlock;
   status += prob;
-  if (tid == 0) {
+  if (tid < 32) {                                      // indices of the active columns, in order
     int na = 0;
-    for (int i = 0; i < m; ++i) if (mask[i]) sh.idx[na++] = i;
-    sh.flag = na;
+    for (int i0 = 0; i0 < m; i0 += 32) {
+      const int i = i0 + tid;
+      const bool on = i < m && mask[i];
+      const unsigned b = __ballot_sync(0xffffffffu, on);
+      if (on) sh.idx[na + __popc(b & ((1u << tid) - 1u))] = i;
+      na += __popc(b);
+    }
+    if (tid == 0) sh.flag = na;
   }
   __syncthreads();
   const int na = sh.flag;
