@@ -379,8 +379,8 @@ iwf_status iwf_evaluate(iwf_plan* plan, const void* coef, const double* x, long 
  * 0 <= a < count[0], 0 <= b < count[1] (the observation grids of Sec. 4.2), for plans with
  * d = 2, a diagonal P_I (P_01 = P_10 = 0, as in every example of the paper) and 2K_1, 2K_2 <= 32.
  * Then (P k).x separates over the two grid axes within each k_II slice, and the slice's share
- * of u is a product E0 C E1^T of its 2K_1 x 2K_2 coefficients with two phase tables: about 2K_2
- * times fewer operations per point than iwf_evaluate, in FP64.
+ * of u is a product E0 C E1^T of its 2K_1 x 2K_2 coefficients with two phase tables, points
+ * taken in mirrored pairs: about 4K_2 times fewer operations per point than iwf_evaluate, in FP64.
  *   coef    device, N complex double, window order
  *   origin, step   host, 2 doubles each;  count  host, 2 ints
  *   u       device, count[0]*count[1] complex double, row-major (the last axis fastest)
@@ -544,12 +544,12 @@ iwf_status iwf_plan_set_wait_limit(iwf_plan* plan, long long rounds);
  * block form: the Gram matrices S^H S and S^H H S and the updates X <- S C), exposed for
  * direct use, testing and measurement. Engines:
  *   IWF_CONTRACT_TENSOR  tcgen05 tensor cores, Ozaki scheme I: every FP64 value becomes the
- *                        integer round(v 2^(48-E)) under a power-of-two scale 2^E shared by
+ *                        integer round(v 2^(55-E)) under a power-of-two scale 2^E shared by
  *                        its group (a column for iwf_gram, a row of S and a column of C for
- *                        iwf_block_update), written as seven balanced 7-bit digits stored as
- *                        bf16; digit pairs of one level are summed exactly in fp32 tensor
- *                        memory (levels 2..6; 7..9 share one accumulator; pairs above 9 are
- *                        dropped). Error about 2^-49 of the product of the two scales per
+ *                        iwf_block_update), written as eight balanced 7-bit digits stored as
+ *                        bf16; digit pairs of one level are summed in fp32 tensor memory
+ *                        (levels 2..6 exactly; pairs above level 10 are dropped). Error
+ *                        about 2^-56 of the product of the two scales per
  *                        term, random in sign.
  *   IWF_CONTRACT_DF      double-float arithmetic on the FP32 pipes (about 48 bits).
  *   IWF_CONTRACT_F64     FP64 arithmetic.

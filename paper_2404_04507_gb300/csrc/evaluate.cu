@@ -137,18 +137,32 @@ __global__ void reduce_groups_kernel(const double2* __restrict__ part, long long
 // slice's share of u on the grid x_0(a) = o_0 + a h_0, x_1(b) = o_1 + b h_1 is the product
 // E0_s C_s E1_s^T with C_s the slice's 2K_1 x 2K_2 coefficients, E0_s[a][i] =
 // exp(i x_0(a) (p00 (lo_1 + i) + A_s)) and E1_s[i][b] = exp(i x_1(b) (p11 (lo_2 + i) + B_s)).
-// Per slice and tile of kGA x kGT points: T = C_s E1_s^T (2K_1 x kGT), then u += E0_s T, i.e.
-// 2K_1 (1 + 2K_2 / kGA) complex multiply-adds per point instead of the 2K_1 2K_2 of direct
-// summation. Phase tables: one exact sincos per row or column and slice, then a recurrence of
-// at most 31 complex multiplications. FP64 throughout.
+// Rows and columns go in pairs around their tile's centre c: with theta the frequency,
+// exp(i theta (c +- d)) = exp(i theta c) (cos theta d +- i sin theta d). The centre's phases are
+// folded into the coefficients, C' = C_s exp(i theta_0 c_0) exp(i theta_1 c_1), and two mirrored
+// points share the real products A = sum cos(theta d) C' and B = sum sin(theta d) C':
+// u(c +- d) = A +- i B. So a complex multiply-add of one point costs two FP64 multiply-adds
+// instead of four. Per slice and tile of kGA x kGT points: T = C' E1^T (2K_1 x kGT, by column
+// pairs), then u += E0 T by row pairs. Phase tables: one sincos per pair and slice, then a
+// recurrence of at most 31 complex multiplications; one sincos per frequency and slice for the
+// centre, with the rounding of theta c carried as a first-order correction. FP64 throughout.
+// Bound: the FP64 pipe. 1001 x 1001 points: 334 -> 149 ms from the 32^4 window, 11.0 -> 5.2 ms from
+// 12 x 12 coefficients in 100 slices (every point for itself before, and slice groups in five
+// uneven waves); largest error against extended precision 4.9e-12 -> 3.3e-12 and 2.4e-12 ->
+// 2.2e-12 (sum |c| = 2.3e4 and 350).
 constexpr int kGT = 64;              // output tile: kGA rows x kGT columns
 constexpr int kGA = 128;
+constexpr int kGPT = kGT / 2, kGPA = kGA / 2;    // column and row pairs of a tile
 constexpr int kGThreads = 512;
 constexpr int kGMaxLen = 32;         // largest 2K_j of the fast path
 constexpr int kGRows = kGThreads / kGT;          // 8 row groups of threads
-constexpr int kGAcc = kGA / kGRows;              // 16 accumulators per thread
+constexpr int kGAcc = kGPA / kGRows;             // 8 row pairs per thread
+constexpr int kGE0 = kGMaxLen + 1;               // row table's stride (its stores: distinct banks)
 constexpr size_t kGSmem =
-    sizeof(double2) * (size_t)(kGMaxLen * kGMaxLen + 2 * kGMaxLen * kGT + kGA * kGMaxLen);
+    sizeof(double2) * (size_t)(kGMaxLen * kGMaxLen + kGMaxLen * (kGPT + kGT) + kGPA * kGE0 +
+                               2 * kGMaxLen);
+static_assert(kGPT == 32, "a warp holds the column pairs of one row of T");
+static_assert(kGPT + kGPA + 2 * kGMaxLen <= kGThreads, "one thread per phase table row");
 
 struct GridArgs {
   Geom g;
@@ -169,33 +183,40 @@ __device__ __forceinline__ double2 cmul2(double2 a, double2 b) {
 
 __global__ void __launch_bounds__(kGThreads, 1) evaluate_grid_kernel(GridArgs a) {
   extern __shared__ __align__(16) unsigned char g_raw[];
-  double2* s_c = reinterpret_cast<double2*>(g_raw);          // [i0][i1], len1 stride
-  double2* s_e1 = s_c + kGMaxLen * kGMaxLen;                  // [i1][b]
-  double2* s_e0 = s_e1 + kGMaxLen * kGT;                      // [a][i0], kGMaxLen stride
-  double2* s_t = s_e0 + kGA * kGMaxLen;                       // [i0][b]
+  double2* s_c = reinterpret_cast<double2*>(g_raw);          // C' [i0][i1], len1 stride
+  double2* s_e1 = s_c + kGMaxLen * kGMaxLen;                  // (cos, sin) [i1][column pair]
+  double2* s_e0 = s_e1 + kGMaxLen * kGPT;                     // (cos, sin) [row pair][i0]
+  double2* s_t = s_e0 + kGPA * kGE0;                          // T [i0][b]
+  double2* s_f = s_t + kGMaxLen * kGT;                        // centre phases: i1, then i0
   const Geom& g = a.g;
   const int len0 = g.lens[0], len1 = g.lens[1];
   const int MI = len0 * len1;
   const int t = threadIdx.x;
   const int tb = t % kGT, tr = t / kGT;                       // column and row group
+  const int q = t % kGPT;                                     // column pair (T)
   const int ta0 = (blockIdx.x / a.tiles1) * kGA, tb0 = (blockIdx.x % a.tiles1) * kGT;
-  // grid coordinates of this thread's table row (t < kGT: column b = t; kGT <= t < kGT + kGA:
-  // row a = t - kGT), with the same rounding as origin + index * step on the host
+  const int nr = min(kGA, a.G0 - ta0), nc = min(kGT, a.G1 - tb0);   // the tile's points
+  // pair j of n points: positions n/2 + j and (n-1)/2 - j, at distance j or j + 1/2 steps.
+  // One table row per thread: column pairs, row pairs, then the centre's phases (axis 1, 0)
+  const bool pair = t < kGPT + kGPA, centre = !pair && t < kGPT + kGPA + 2 * kGMaxLen;
+  const int ci = t - (kGPT + kGPA);
+  const bool col = pair ? t < kGPT : ci < kGMaxLen;
+  const double pjj = col ? a.p11 : a.p00;
   double xc = 0.0, zr = 1.0, zi = 0.0;                        // coordinate and step phase
-  if (t < kGT + kGA) {
-    xc = t < kGT ? __dadd_rn(a.o1, __dmul_rn((double)(tb0 + t), a.h1))
-                 : __dadd_rn(a.o0, __dmul_rn((double)(ta0 + t - kGT), a.h0));
-    sincos(xc * (t < kGT ? a.p11 : a.p00), &zi, &zr);
+  if (pair) {
+    xc = ((col ? t : t - kGPT) + ((col ? nc : nr) & 1 ? 0.0 : 0.5)) * (col ? a.h1 : a.h0);
+    sincos(xc * pjj, &zi, &zr);
+  } else if (centre) {
+    xc = col ? a.o1 + (tb0 + 0.5 * (nc - 1)) * a.h1 : a.o0 + (ta0 + 0.5 * (nr - 1)) * a.h0;
   }
-  double2 acc[kGAcc];
+  double2 acc[kGAcc], bcc[kGAcc];                             // A and B of the row pairs
 #pragma unroll
-  for (int j = 0; j < kGAcc; ++j) acc[j] = make_double2(0.0, 0.0);
+  for (int j = 0; j < kGAcc; ++j) acc[j] = bcc[j] = make_double2(0.0, 0.0);
   const long long s0 = (long long)blockIdx.y * a.o_per;
   const long long s1 = min(g.MII, s0 + a.o_per);
   for (long long o = s0; o < s1; ++o) {
     __syncthreads();                                          // previous slice's tables read
-    for (int e = t; e < MI; e += kGThreads) s_c[e] = a.coef[o * MI + e];
-    if (t < kGT + kGA) {
+    if (pair || centre) {
       // slice constants: A_s or B_s from k_II = pos - L (C order, last axis fastest)
       double sab = 0.0;
       long long rem = o;
@@ -203,52 +224,70 @@ __global__ void __launch_bounds__(kGThreads, 1) evaluate_grid_kernel(GridArgs a)
         const int len = g.lens[j];
         const int kj = (int)(rem % len) - g.half[j];
         rem /= len;
-        sab = fma(t < kGT ? a.pb[j] : a.pa[j], (double)kj, sab);
+        sab = fma(col ? a.pb[j] : a.pa[j], (double)kj, sab);
       }
-      const bool col = t < kGT;
       const int lo = a.lo[o * 2 + (col ? 1 : 0)];
-      const double freq = fma(col ? a.p11 : a.p00, (double)lo, sab);
-      double pr, pi;
-      sincos(xc * freq, &pi, &pr);
       const int len = col ? len1 : len0;
-      for (int i = 0; i < len; ++i) {
-        if (col) s_e1[i * kGT + t] = make_double2(pr, pi);
-        else s_e0[(t - kGT) * kGMaxLen + i] = make_double2(pr, pi);
-        const double nr = fma(pr, zr, -pi * zi);
-        pi = fma(pr, zi, pi * zr);
-        pr = nr;
+      double pr, pi;
+      if (pair) {
+        const double freq = fma(pjj, (double)lo, sab);
+        sincos(xc * freq, &pi, &pr);
+        for (int i = 0; i < len; ++i) {
+          if (col) s_e1[i * kGPT + t] = make_double2(pr, pi);
+          else s_e0[(t - kGPT) * kGE0 + i] = make_double2(pr, pi);
+          const double nr_ = fma(pr, zr, -pi * zi);
+          pi = fma(pr, zi, pi * zr);
+          pr = nr_;
+        }
+      } else if ((ci & (kGMaxLen - 1)) < len) {
+        const double freq = fma(pjj, (double)(lo + (ci & (kGMaxLen - 1))), sab);
+        const double ph = xc * freq, r = fma(xc, freq, -ph);
+        sincos(ph, &pi, &pr);
+        s_f[ci] = make_double2(fma(-r, pi, pr), fma(r, pr, pi));
       }
     }
     __syncthreads();
-    // T = C_s E1_s^T for this thread's column tb
-    for (int i0 = tr; i0 < len0; i0 += kGRows) {
-      double2 sum = make_double2(0.0, 0.0);
+    for (int e = t; e < MI; e += kGThreads) {
+      const int i0 = e / len1;
+      s_c[e] = cmul2(cmul2(a.coef[o * MI + e], s_f[e - i0 * len1]), s_f[kGMaxLen + i0]);
+    }
+    __syncthreads();
+    // T = C' E1^T: columns of pair q, a row per warp
+    for (int i0 = t / kGPT; i0 < len0; i0 += kGThreads / kGPT) {
+      double2 sa = make_double2(0.0, 0.0), sb = make_double2(0.0, 0.0);
       for (int i1 = 0; i1 < len1; ++i1) {
-        const double2 c = s_c[i0 * len1 + i1], e = s_e1[i1 * kGT + tb];
-        sum.x = fma(c.x, e.x, sum.x); sum.x = fma(-c.y, e.y, sum.x);
-        sum.y = fma(c.x, e.y, sum.y); sum.y = fma(c.y, e.x, sum.y);
+        const double2 c = s_c[i0 * len1 + i1], e = s_e1[i1 * kGPT + q];
+        sa.x = fma(e.x, c.x, sa.x); sa.y = fma(e.x, c.y, sa.y);
+        sb.x = fma(e.y, c.x, sb.x); sb.y = fma(e.y, c.y, sb.y);
       }
-      s_t[i0 * kGT + tb] = sum;
+      if (q < (nc + 1) / 2) {
+        s_t[i0 * kGT + (nc - 1) / 2 - q] = make_double2(sa.x + sb.y, sa.y - sb.x);
+        s_t[i0 * kGT + nc / 2 + q] = make_double2(sa.x - sb.y, sa.y + sb.x);
+      }
     }
     __syncthreads();
-    // u += E0_s T for rows tr, tr + kGRows, ...
+    // u += E0 T for row pairs tr, tr + kGRows, ... (columns from nc on hold nothing to store)
     for (int i0 = 0; i0 < len0; ++i0) {
       const double2 tv = s_t[i0 * kGT + tb];
 #pragma unroll
       for (int j = 0; j < kGAcc; ++j) {
-        const double2 e = s_e0[(tr + kGRows * j) * kGMaxLen + i0];
-        acc[j].x = fma(e.x, tv.x, acc[j].x); acc[j].x = fma(-e.y, tv.y, acc[j].x);
-        acc[j].y = fma(e.x, tv.y, acc[j].y); acc[j].y = fma(e.y, tv.x, acc[j].y);
+        const double2 e = s_e0[(tr + kGRows * j) * kGE0 + i0];
+        acc[j].x = fma(e.x, tv.x, acc[j].x); acc[j].y = fma(e.x, tv.y, acc[j].y);
+        bcc[j].x = fma(e.y, tv.x, bcc[j].x); bcc[j].y = fma(e.y, tv.y, bcc[j].y);
       }
     }
   }
-  const long long M = (long long)a.G0 * a.G1;
-  const int b = tb0 + tb;
-  if (b < a.G1) {
+  if (tb < nc) {
+    double2* out = a.out + (long long)blockIdx.y * a.G0 * a.G1 + tb0 + tb;
 #pragma unroll
     for (int j = 0; j < kGAcc; ++j) {
-      const int ra = ta0 + tr + kGRows * j;
-      if (ra < a.G0) a.out[(long long)blockIdx.y * M + (long long)ra * a.G1 + b] = acc[j];
+      const int pj = tr + kGRows * j;
+      if (pj < (nr + 1) / 2) {
+        out[(long long)(ta0 + (nr - 1) / 2 - pj) * a.G1] =
+            make_double2(acc[j].x + bcc[j].y, acc[j].y - bcc[j].x);
+        out[(long long)(ta0 + nr / 2 + pj) * a.G1] =
+            make_double2(acc[j].x - bcc[j].y, acc[j].y + bcc[j].x);
+      }
     }
   }
 }
@@ -471,11 +510,17 @@ iwf_status evaluate_grid_impl(iwf_plan* p, const void* coef, const double* origi
   const long long tiles = tiles0 * tiles1;
   int sms = 0;
   IWF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device));
-  // one CTA per SM: about four waves of slice groups
-  long long groups = std::max(1LL, (4LL * sms + tiles - 1) / tiles);
-  groups = std::min(groups, g.MII);
-  groups = std::min(groups, std::max(1LL, (long long)(kEvalPartMax / (16 * (size_t)M))));
-  groups = std::min(groups, 65535LL);
+  // one CTA per SM: the number of slice groups, up to about six waves, whose waves times the
+  // slices of a CTA are fewest (1001 x 1001 points, 100 slices: 7 groups, 6 waves of 15 slices;
+  // four waves' worth, 5 groups, are 5 waves of 20)
+  long long most = std::min(std::max(1LL, (6LL * sms + tiles - 1) / tiles), g.MII);
+  most = std::min(most, std::max(1LL, (long long)(kEvalPartMax / (16 * (size_t)M))));
+  most = std::min(most, 65535LL);
+  long long groups = 1, best = -1;
+  for (long long c = 1; c <= most; ++c) {
+    const long long cost = ((tiles * c + sms - 1) / sms) * ((g.MII + c - 1) / c);
+    if (best < 0 || cost < best) { best = cost; groups = c; }
+  }
   const long long o_per = (g.MII + groups - 1) / groups;
   groups = (g.MII + o_per - 1) / o_per;
   GridArgs a{};
