@@ -49,7 +49,7 @@ PASS_B_KERNEL = {"pencil": "pencil_b_kernel<double,32,4>", "tiled": "pass_kernel
 PROFILE_FILE = os.path.join(ROOT, "profiles", "pencil_pass_b_moire32_f64.txt")
 # the schedule the autotuner picks for this workload on a GB300 (threads, tile KB, chunk MB);
 # --fixed-schedule applies it without tuning, so profiler runs see only the timed kernels
-FIXED_SCHEDULE = {"f64": (128, 96, 96, "pencil"), "c64": (128, 96, 48, "pencil")}
+FIXED_SCHEDULE = {"f64": (128, 96, 96, "auto"), "c64": (128, 96, 48, "auto")}
 
 
 def _dist():
@@ -135,6 +135,19 @@ def pass_b_flops_per_point(lens, d) -> float:
     """Pass B: inverse + forward DFT along the k_II axes (5 log2 M_II each) and V (2 flops)."""
     mii = float(np.prod(lens[d:]))
     return 10.0 * math.log2(mii) + 2.0
+
+
+def direct_flops_per_point(pb, lens) -> float:
+    """Flops per point and vector of the direct convolution: a multiply-add per real and imaginary
+    part for Lambda and for every folded mode but the constant (twice that for a complex
+    coefficient)."""
+    modes = {}
+    for m, c in zip(pb.modes, pb.coef):
+        k = tuple(int(v) % int(n) for v, n in zip(m, lens))
+        modes[k] = modes.get(k, 0.0) + c
+    modes.pop((0,) * len(lens), None)
+    real = all(c.imag == 0.0 for c in modes.values())
+    return 4.0 + (4.0 if real else 8.0) * len(modes)
 
 
 def _source_hash() -> str:
@@ -664,7 +677,20 @@ def run_ours(args):
     pts = float(N) * NVEC
     value = pts * ws / (ms * 1e-3)
 
-    # dominant kernel (pass B) per-launch duration, events on the launching stream
+    # one launch a step: the direct convolution, bound by the FP64 pipe; its own roofline
+    direct = launches == args.steps
+    direct_roofline = None
+    if direct:
+        tf = direct_flops_per_point(pb, plan.lens) * pts / (ms * 1e-3) / 1e12
+        direct_roofline = {"bound": "alu", "achieved": tf, "peak": FP64_PEAK_TFLOPS,
+                           "unit": "TFLOP/s", "frac": tf / FP64_PEAK_TFLOPS, "traffic": None,
+                           "kernel": "direct_kernel<double,2,4,4,true> (whole apply)",
+                           "frac_of_measured_fp64": tf / FP64_MEASURED_TFLOPS,
+                           "launch_ms": ms,
+                           "algorithmic_flops": f"{direct_flops_per_point(pb, plan.lens):.0f} "
+                                                "per point and vector"}
+
+    # the transforms' pass B, per-launch duration, events on the launching stream
     pass_ms, pass_n = np.zeros(3), np.zeros(3)
     nprof = max(3, args.steps // 2)
     for _ in range(nprof):
@@ -686,6 +712,9 @@ def run_ours(args):
                 "frac_of_measured_fp64": achieved / FP64_MEASURED_TFLOPS,
                 "vectors_per_launch": chunk, "launch_ms": per_launch[1],
                 "pass_ms_share": (pass_ms / pass_ms.sum()).round(4).tolist()}
+    ms_transforms = pass_ms.sum() / nprof
+    if direct:
+        roofline = dict(direct_roofline, transforms=dict(roofline, ms_per_apply=ms_transforms))
 
     # complex64 apply of the same block (the mixed-precision path), HBM-bound
     xc = x.to(torch.complex64)
@@ -714,13 +743,14 @@ def run_ours(args):
            "roofline": {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s",
                         "frac": gbs / hbm, "traffic": None, "of": "measured",
                         "algorithmic_bytes": "16 B per point and vector (read psi, write H psi)",
-                        "note": "whole three-pass apply: the block is read and written once per "
+                        "note": "direct convolution: one pass" if direct else
+                                "whole three-pass apply: the block is read and written once per "
                                 "pass and psi is read again by pass C"}}
 
     # the same FP64 apply with double-float DFTs (IWF_ARITH_DF, pencil path): storage, the
     # potential and the kinetic term stay FP64, the DFTs run on the FP32 pipes
     df_apply = None
-    if tune["f64"]["path"] == "pencil":
+    if tune["f64"]["path"] in ("auto", "pencil"):
         plan.set_arith("df")
         yd = torch.empty_like(x)
         for _ in range(3):
@@ -742,12 +772,12 @@ def run_ours(args):
         plan.apply(x, y)
         diff = float(((yd - y).abs().max() / y.abs().max()).item())
         df_apply = {"value": pts / (ms_df * 1e-3), "unit": UNIT, "ms_per_step": ms_df,
-                    "speedup_vs_fp64_dfts": ms / ms_df, "max_rel_diff_vs_fp64_dfts": diff,
+                    "speedup_vs_fp64_dfts": ms_transforms / ms_df, "max_rel_diff_vs_fp64_dfts": diff,
                     "pass_ms_per_apply": (d_ms / 3).round(4).tolist(),
                     "arith": "double-float DFTs (about 48 significant bits) on the FP32 pipes; "
                              "FP64 storage, potential tables and kinetic term"}
 
-    # ablation: the same operator by direct convolution with the potential's 8 folded modes
+    # the same operator by iwf_apply_stencil: direct convolution with the potential's 8 folded modes
     # (iwf_apply_stencil), both precisions, against HBM (one read, one write per point)
     stencil = {}
     nmodes_folded = len({tuple(int(v) % int(L) for v, L in zip(m, plan.lens)) for m in pb.modes})
@@ -767,16 +797,17 @@ def run_ours(args):
                 "frac": gbs_s / hbm, "of": "measured",
                 "algorithmic_bytes": f"{int(elt)} B per point and vector"}
         if name == "f64":
-            # FP64 ALU bound: one complex multiply-add (8 flops) per mode + Lambda psi (2)
-            tf = (8.0 * nmodes_folded + 2.0) * pts / (ms_s * 1e-3) / 1e12
+            # FP64 ALU bound
+            fl = direct_flops_per_point(pb, plan.lens)
+            tf = fl * pts / (ms_s * 1e-3) / 1e12
             roof = {"bound": "alu", "achieved": tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                     "frac": tf / FP64_PEAK_TFLOPS,
-                    "algorithmic_flops": f"{8 * nmodes_folded + 2} per point and vector",
+                    "algorithmic_flops": f"{fl:.0f} per point and vector",
                     "hbm_gbs": gbs_s}
         stencil[name] = {"value": pts / (ms_s * 1e-3), "unit": UNIT, "ms_per_step": ms_s,
                          "roofline": roof}
-    stencil["note"] = (f"ablation, not the product path: direct convolution with the "
-                       f"{nmodes_folded} folded modes; its cost grows with the number of modes")
+    stencil["note"] = (f"direct convolution with the {nmodes_folded} folded modes (what apply() takes "
+                       f"for few modes); its cost grows with the number of modes")
 
     # axes above 32 (shared-memory FFT, pass_long_kernel): the FP64 apply of a 16-vector
     # block on the reference window of the paper's 1D accuracy table, Example 4.1 with PM
@@ -799,7 +830,7 @@ def run_ours(args):
         torch.cuda.synchronize()
         ms_l = e0.elapsed_time(e1) / nrep
         lpts = float(lplan.N) * NVEC
-        lflops = 10.0 * math.log2(lplan.N) + 6.0
+        lflops = direct_flops_per_point(pl, lplan.lens)   # (the autotuner keeps the direct apply)
         tf_l = lflops * lpts / (ms_l * 1e-3) / 1e12
         l_ms, l_n = np.zeros(3), np.zeros(3)
         for _ in range(3):
@@ -811,8 +842,7 @@ def run_ours(args):
                      "pass_ms_per_apply": (l_ms / 3).round(4).tolist(),
                      "roofline": {"bound": "alu", "achieved": tf_l, "peak": FP64_PEAK_TFLOPS,
                                   "unit": "TFLOP/s", "frac": tf_l / FP64_PEAK_TFLOPS,
-                                  "algorithmic_flops": f"{lflops:.0f} per point and vector "
-                                                       "(10 log2 N + 6)"}}
+                                  "algorithmic_flops": f"{lflops:.0f} per point and vector"}}
         lplan.close()
         del lx, ly
 
@@ -849,7 +879,7 @@ def run_ours(args):
         ms_grid = e0.elapsed_time(e1)
         L0, L1 = plan.lens[0], plan.lens[1]
         mii = plan.N // (L0 * L1)
-        gflops = 8.0 * mii * L0 * gcount[1] * (L1 + gcount[0])
+        gflops = 4.0 * mii * L0 * gcount[1] * (L1 + gcount[0])   # points in mirrored pairs
         tf_grid = gflops / (ms_grid * 1e-3) / 1e12
         del ug
         terms = float(M) * plan.N
@@ -864,7 +894,7 @@ def run_ours(args):
                      "ms": ms_grid, "speedup_vs_direct": ms_ev * 1001 / args.eval_rows / ms_grid,
                      "roofline": {"bound": "alu", "achieved": tf_grid, "peak": FP64_PEAK_TFLOPS,
                                   "unit": "TFLOP/s", "frac": tf_grid / FP64_PEAK_TFLOPS,
-                                  "algorithmic_flops": "8 MII 2K_1 G_1 (2K_2 + G_0): the two "
+                                  "algorithmic_flops": "4 MII 2K_1 G_1 (2K_2 + G_0): the two "
                                                        "products per slice"}},
             "roofline": {"bound": "alu", "achieved": tf_ev, "peak": FP64_PEAK_TFLOPS,
                          "unit": "TFLOP/s", "frac": tf_ev / FP64_PEAK_TFLOPS,

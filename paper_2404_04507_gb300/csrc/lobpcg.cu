@@ -358,8 +358,8 @@ iwf_status run_phase(iwf_plan* p, const ApplyBatch* ab, int b, int nev, int maxi
 
 // ---- returned eigenvalues: FP64 Rayleigh quotients of the returned vectors ----
 // theta_j = Re(x_j^H (H x)_j) / (x_j^H x_j) with H x applied afresh. The Ritz values of the
-// double-float Rayleigh-Ritz carry its rounding (a few 1e-12 when the projected matrix has
-// large entries); these quotients carry only FP64 rounding of two dot products and of one
+// Rayleigh-Ritz step carry the rounding of its projected matrix (whose entries grow with the
+// largest Lambda in the basis); these quotients carry only FP64 rounding of two dot products and of one
 // apply, and differ from the exact eigenvalue by O(residual^2 / gap).
 constexpr int kRqThreads = 256;
 
