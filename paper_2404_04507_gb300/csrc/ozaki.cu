@@ -934,14 +934,14 @@ iwf_status launch_gram_tc(const Batch& bt, const BlockList& A, const BlockList& 
   int S = kMaxStages;
   while (S > 2 && Lo.smem(S) > kSmemCap) --S;
   if (Lo.smem(S) > kSmemCap) return fail(IWF_ERR_ARG, "gram_tc: tiles exceed shared memory");
-  // rows per CTA: whole accumulation chunks for long blocks; for short ones as few stages as give
-  // every SM a CTA (14400 and 20736 rows: whole chunks left 28 and 41 CTAs; 20736 x 24, 45 -> 22 us)
+  // rows per CTA: as few stages as give every SM a CTA. Whole accumulation chunks of 512 rows left 28
+  // and 41 CTAs at 14400 and 20736 rows (20736 x 24: 45 us, now 22) and four chunks for 115 CTAs
+  // where three and a bit for 152 do at 234256 (48 x 24 columns: 176 us, now 145).
   long long want = std::max(1, sm_count() / (subs.n * std::max(1, bt.nprob)));
   want = std::min<long long>(want, std::max<long long>(
                                        1, partial_cap / ((long long)subs.slot_size * bt.nprob)));
-  const long long unit = N >= want * kChunkRows ? kChunkRows : kStageRows;
-  const long long units = (N + unit - 1) / unit;
-  const long long per = (units + want - 1) / want * unit;
+  const long long stages = (N + kStageRows - 1) / kStageRows;
+  const long long per = (stages + want - 1) / want * kStageRows;
   const int slots = (int)((N + per - 1) / per);
   dim3 grid((unsigned)std::max(1, slots), (unsigned)bt.nprob, (unsigned)subs.n);
   gram_tc_kernel<NMMA><<<grid, kGramThreads, Lo.smem(S), s>>>(bt, A, B, N, per, S, subs, partial,
