@@ -105,17 +105,18 @@ template <bool REAL> struct ModeSum<float, REAL> {
 // Measured on 16 vectors, transforms before and this kernel now: complex double, 32^4, 8 real
 // modes 4330 -> 514 us (bound by the FP64 pipe: 18 operations a point, 480 us at its peak), Example
 // 4.1's 1280 x 2048 23.85 -> 0.74 ms (also FP64); complex float, 32^4, 8 complex modes 184 ->
-// 98 us, 8 real ones 91 us, 16^6, 12 modes 15.1 -> 1.5 ms (issue and L1 latency together; ncu at 32^4: issue 51 %,
+// 92 us, 16^6, 12 modes 15.1 -> 1.5 ms (issue and L1 latency together; ncu at 32^4: issue 51 %,
 // L1 50 %, DRAM 30 %, L2 29 %). NV = 2 or 8 were 30 % slower in complex float (index arithmetic;
 // registers), U = 2 slower on 16^6, and patches of 2 x 2 to 4 x 8 slices a CTA, so that neighbour
 // slices come from its own L1, no faster anywhere. psi itself is loaded after the modes: held in
 // registers meanwhile it costs occupancy (111 us). Complex
 // float runs with register bounds, none of which spills: three k_I axes for five CTAs an SM (16^6:
-// 1.50 against 1.94 ms), the others for three (8 complex modes at 32^4 98 against 125 us with 92
-// registers, 22^4, 24 vectors 45 against 55 us, 1280 x 2048 185 against 446 us with 175).
+// 1.50 against 1.94 ms), two for four (8 complex modes at 32^4 92 us, 98 with three CTAs, 125 with
+// the two that 92 registers allow; 22^4, 24 vectors 41, 45 and 55 us), the others for three, since
+// four spill (1280 x 2048 185 against 446 us with one, at 175 registers).
 // D: number of k_I axes when it is 1, 2 or 3; 0 handles any d. REAL: every coefficient is real.
 template <typename T, int D, int NV, int U, bool REAL>
-__global__ void __launch_bounds__(kDirectThreads, sizeof(T) == 8 ? 1 : D == 3 ? 5 : 3)
+__global__ void __launch_bounds__(kDirectThreads, sizeof(T) == 8 ? 1 : D == 3 ? 5 : D == 2 ? 4 : 3)
 direct_kernel(DirectArgs a) {
   using V2 = typename SVec2<T>::type;
   using Off = typename std::conditional<(D > 0), unsigned, size_t>::type;  // byte offsets
