@@ -44,6 +44,7 @@ struct DirectArgs {
   int groups;             // vector groups of a problem
   const int* active;      // problem p skipped when active[p] == 0 (may be null)
   int S, P;               // slices per CTA, threads per slice
+  int parts;              // CTAs that share a slice (1 when S > 1)
   unsigned mag1, mag2;    // ceil(2^32 / len) of the faster k_I axes
 };
 
@@ -98,10 +99,11 @@ template <bool REAL> struct ModeSum<float, REAL> {
   }
 };
 
-// CTA: blockIdx.x = S neighbouring slices (one, unless slices are smaller than a CTA),
-// blockIdx.y = (problem, group of NV vectors). Thread (s, t) owns positions t, t + P, ... of
-// slice s in NV vectors, so that a mode's index arithmetic is paid once for NV vectors; the
-// neighbours of U modes are loaded before they are used.
+// CTA: blockIdx.x = S neighbouring slices (one, unless slices are smaller than a CTA), or one of
+// `parts` shares of a slice where there are few slices; blockIdx.y = (problem, group of NV vectors).
+// Thread (s, t) owns positions t, t + P, ... of slice s (with parts, every parts-th run of P) in NV
+// vectors, so that a mode's index arithmetic is paid once for NV vectors; the neighbours of U modes
+// are loaded before they are used.
 // Measured on 16 vectors, transforms before and this kernel now: complex double, 32^4, 8 real
 // modes 4330 -> 514 us (bound by the FP64 pipe: 18 operations a point, 480 us at its peak), Example
 // 4.1's 1280 x 2048 23.85 -> 0.74 ms (also FP64); complex float, 32^4, 8 complex modes 184 ->
@@ -130,7 +132,8 @@ direct_kernel(DirectArgs a) {
   V2* s_c = reinterpret_cast<V2*>(smem_raw);
   int* s_m = reinterpret_cast<int*>(smem_raw + (size_t)((nm + 1) & ~1) * sizeof(V2));
   const int MI = (int)g.MI;
-  const int o0 = blockIdx.x * S;
+  const int run = blockIdx.x % (unsigned)a.parts;
+  const int o0 = (int)(blockIdx.x / (unsigned)a.parts) * S;
   for (int e = threadIdx.x; e < nm * S; e += blockDim.x) {
     const int q = e / S, o = o0 + e - q * S;
     if (o >= g.MII) continue;
@@ -174,7 +177,7 @@ direct_kernel(DirectArgs a) {
     base[v] = reinterpret_cast<const char*>(a.psi) + (size_t)(v0 + min(v, nv - 1)) * a.ld * sizeof(V2);
   const auto load = [&](int v, Off i) { return __ldg(reinterpret_cast<const V2*>(base[v] + i)); };
   V2* out = reinterpret_cast<V2*>(a.out) + (size_t)v0 * a.ld + (size_t)o * MI;
-  for (int w = t; w < MI; w += a.P) {
+  for (int w = run * a.P + t; w < MI; w += a.parts * a.P) {
     // coordinates of position w along the k_I axes (C order)
     int w0 = w, w1 = 0, w2 = 0;
     int wc[IWF_MAX_N];
@@ -255,7 +258,16 @@ iwf_status launch_direct(DirectArgs a, bool real, int nprob, cudaStream_t s) {
   using V2 = typename SVec2<T>::type;
   constexpr int U = 4;
   a.groups = (a.vpp + NV - 1) / NV;
-  const long long blocks = (a.g.MII + a.S - 1) / a.S;
+  const long long slices = (a.g.MII + a.S - 1) / a.S;
+  // A slice is shared among CTAs where there are fewer than four an SM: a window of few slices
+  // (8^4 x 16, 48 real modes, 4 vectors: 16 CTAs, 390 us where the transforms take 164) otherwise
+  // leaves the chip idle (now 45 us). With four or more, sharing only repeats the shifts' set-up.
+  int sms = 0, dev = 0;
+  IWF_CUDA(cudaGetDevice(&dev));
+  IWF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const long long want = 4LL * sms / std::max(1LL, slices * nprob * a.groups);
+  a.parts = (int)std::max(1LL, std::min<long long>(want, (a.g.MI + a.P - 1) / a.P));
+  const long long blocks = slices * a.parts;
   if ((long long)nprob * a.groups > 65535 || blocks > 2147483647LL)
     return fail(IWF_ERR_UNSUPPORTED, "direct apply: too many slices or vectors");
   const size_t smem = (size_t)((a.nm + 1) & ~1) * sizeof(V2) +
