@@ -863,19 +863,29 @@ update_tc_kernel(Batch bt, BlockList S, int m, long long N, const double2* C1, c
 #pragma unroll
           for (int w = 0; w < 2; ++w) {
             const int n = 8 * g + u + w;
-            // x 2^42 = the level sums: levels 2..6 are integers below 2^22 in units of
-            // 2^(-7(l-2)), gathered exactly (below 2^62), two of them in 32 bits first; levels
-            // 7..10, together in units of 2^-35, are rounded to 2^-42 (the pairs that are dropped
-            // leave about 2^-48 of a level-2 unit)
+            // Levels 2..6 are integers below 2^22 in units of 2^(-7(l-2)), gathered exactly, two of
+            // them in 32 bits first; levels 7..10, together in units of 2^-35 (and below 2^22 of
+            // them), are an integer, which joins the others in T (below 2^55), and a fraction of
+            // 14 bits. A sum below 2^48 takes the whole fraction, so that what is rounded here lies
+            // below the rounding of levels 7..10 however much has cancelled (rounded to 2^-42 in
+            // every sum, those whose leading bits cancel were off by 16 times as much with one
+            // column, 1.9 times with 72). A larger sum loses at least 9 of the 14 bits to FP64: it
+            // takes 8, the last one set if a bit below it is (the side of a tie).
             const int m12 = magic_int(a[1][u + w]) * 128 + magic_int(a[2][u + w]);
             const int m34 = magic_int(a[3][u + w]) * 128 + magic_int(a[4][u + w]);
             const long long top = (long long)magic_int(a[0][u + w]) * 16384 + m12;
-            const long long T = (((top << 14) + m34) << 14) + __float2int_rn(a[5][u + w] * 128.0f);
-            // value = T 2^-42 2^(Er + En - 12), E = maxb - 1022
+            const float whole = a[5][u + w] + 12582912.0f;
+            const int frac = __float_as_int(fmaf(a[5][u + w] - (whole - 12582912.0f), 16384.0f,
+                                                 12582912.0f)) - 0x4B400000;
+            const long long T = (((top << 14) + m34) << 7) + (__float_as_int(whole) - 0x4B400000);
+            const bool small = (unsigned)((int)(T >> 32) + (1 << 16)) < (1u << 17);
+            const long long U = small ? T * 16384 + frac
+                                      : T * 256 + ((frac >> 6) | ((frac & 63) != 0));
+            // value = U 2^-49 (or 2^-43) 2^(Er + En - 12), E = maxb - 1022
             const int en = colexpB[n];
             val[w] = (er >= 2047 || en >= 2047)
                          ? nan("")
-                         : ll_to_double_scaled(T, er + en - 2044 - 12 - 42);
+                         : ll_to_double_scaled(U, er + en - 2044 - 12 - (small ? 49 : 43));
           }
           double2* dst = Y + (size_t)jc * N + r;
           if (SUB) {
