@@ -611,40 +611,62 @@ __device__ bool inv_sqrt_series(SmallShared& sh, const double2* M, double2* T, d
   return true;
 }
 
-// T (b x b, upper triangular) = R^{-1} for the Cholesky factor M = R^H R of a Hermitian matrix (its
-// upper triangle is read, and overwritten). Columns whose pivot is not above drop depend on the
-// ones before them: their column of T is zero and sh.keep 0. T is built along with the factor,
-// as Gram-Schmidt on the unit vectors: 24 steps of one square root and one update each.
+// T (b x b) for the Cholesky factorisation with diagonal pivoting of a Hermitian matrix M (full,
+// overwritten): T^H M T = I on the columns kept. The largest pivot left comes next, so that columns
+// with a pivot not above drop, which depend on those before them, come last: their column of T is
+// zero and sh.keep 0. Without pivoting small pivots arise early and amplify what follows: columns of
+// a nearly dependent block came out 8e-9 off the space they had been projected out of, where the
+// eigenvectors of M leave 6e-12 and this order 2e-11 (24 powers of x on [0, 1], drop 1e-14 of the
+// largest eigenvalue). T is built along with the factor, as Gram-Schmidt on the unit vectors: 24
+// steps of one square root and one update each. b <= 32.
 __device__ void cholesky_transform(SmallShared& sh, double2* M, double2* T, int b, double drop) {
   const int tid = threadIdx.x;
+  int* perm = sh.idx;                                  // the order of the pivots
   for (int e = tid; e < b * b; e += kSmallThreads) T[e] = make_double2(e / b == e % b ? 1.0 : 0.0, 0.0);
+  for (int k = tid; k < b; k += kSmallThreads) perm[k] = k;
   __syncthreads();
   for (int k = 0; k < b; ++k) {
-    if (tid == 0) {
-      const double piv = M[k * b + k].x;
-      const bool ok = piv > drop;
-      const double r = ok ? rsqrt(piv) : 0.0;
-      sh.scale[k] = r;
-      sh.r2 = r * r;
-      sh.keep[k] = ok;
+    if (tid < 32) {
+      // by the high words, as integers: close enough for an order
+      const int pos = k + tid;
+      const int c = pos < b ? perm[pos] : 0;
+      const int key = pos < b ? max(0, __double2hiint(M[c * b + c].x)) : -1;
+      const int best = __ffs(__ballot_sync(0xffffffffu, key == __reduce_max_sync(0xffffffffu, key))) - 1;
+      if (tid == best) {
+        const double piv = M[c * b + c].x;
+        const bool ok = piv > drop;
+        const double r = ok ? rsqrt(piv) : 0.0;
+        sh.scale[c] = r;
+        sh.r2 = r * r;
+        sh.keep[c] = ok;
+        perm[pos] = perm[k];
+        perm[k] = c;
+      }
     }
     __syncthreads();
-    if (sh.keep[k]) {
+    const int ck = perm[k];
+    if (sh.keep[ck]) {
       const double r2 = sh.r2;
       const int rest = b - 1 - k, tri = rest * (rest + 1) / 2;
       for (int e = tid; e < tri + (k + 1) * rest; e += kSmallThreads) {
         int i, j;
-        if (e < tri) {                                 // M_ij -= conj(M_ki) M_kj / M_kk
+        if (e < tri) {                                 // M_ij -= conj(M_ki) M_kj / M_kk, mirrored
           fold(e, rest, j, i);
           i += k + 1; j += k + 1;
         } else {                                       // T_ij -= T_ik M_kj / M_kk
           i = (e - tri) / rest;
           j = k + 1 + (e - tri) - i * rest;
         }
-        const double2 m = M[k * b + j];
+        const int ci = perm[i], cj = perm[j];
+        const double2 m = M[ck * b + cj];
         const double2 g = make_double2(-m.x * r2, -m.y * r2);
-        if (e < tri) M[i * b + j] = cmac_conj(M[k * b + i], g, M[i * b + j]);
-        else T[i * b + j] = cmac(T[i * b + k], g, T[i * b + j]);
+        if (e < tri) {
+          const double2 u = cmac_conj(M[ck * b + ci], g, M[ci * b + cj]);
+          M[ci * b + cj] = u;
+          if (ci != cj) M[cj * b + ci] = make_double2(u.x, -u.y);
+        } else {
+          T[ci * b + cj] = cmac(T[ci * b + ck], g, T[ci * b + cj]);
+        }
       }
     }
     __syncthreads();
@@ -659,9 +681,11 @@ __device__ void cholesky_transform(SmallShared& sh, double2* M, double2* T, int 
 // Orthonormalising transform of a block Y from its Gram matrix: Y T is orthonormal on the columns
 // that are kept; dependent columns of T are zero with their mask entry 0. With D =
 // diag(G)^{-1/2}: T = D (D G D)^{-1/2} from its series when the block is orthonormal up to 1e-6
-// already, else D R^{-1} with the Cholesky factor R of D G D, which costs a tenth of the
-// eigenproblem of SVQB (25 against 220 us at b = 24). As there, a second application to the result
-// removes the rounding that small pivots amplify.
+// already, else from the pivoted Cholesky factorisation of D G D, which costs a fraction of the
+// eigenproblem of SVQB (41 against 617 us at b = 24, 10 against 78 at 4). Dependent are columns whose pivot is at most drop times a bound of the
+// largest eigenvalue (the largest absolute row sum), which takes the place of SVQB's test of the
+// eigenvalues. As there, a second application to the result removes the rounding that small pivots
+// amplify.
 __global__ void __launch_bounds__(kSmallThreads, 1)
 svqb_kernel(Batch bt, const double2* G, int b, double drop, double2* T, int* mask, int* status) {
   extern __shared__ __align__(16) unsigned char raw[];
@@ -687,7 +711,19 @@ svqb_kernel(Batch bt, const double2* G, int b, double drop, double2* T, int* mas
   }
   __syncthreads();
   const bool series = inv_sqrt_series(sh, sh.A, sh.B, sh.V, b, D);
-  if (!series) cholesky_transform(sh, sh.A, sh.B, b, drop);
+  if (!series) {
+    if (tid == 0) sh.flag = 0;
+    __syncthreads();
+    for (int i = tid >> 5; i < b; i += kSmallThreads / 32) {
+      const int j = tid & 31;
+      const double2 v = j < b ? sh.A[i * b + j] : make_double2(0.0, 0.0);
+      float r = fabsf((float)v.x) + fabsf((float)v.y);
+      for (int o = 16; o; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+      if (j == 0 && r < 1e3f) atomicMax(&sh.flag, __float_as_int(r));
+    }
+    __syncthreads();
+    cholesky_transform(sh, sh.A, sh.B, b, drop * (double)__int_as_float(sh.flag));
+  }
   for (int e = tid; e < b * b; e += kSmallThreads) {
     const double f = D[e / b];
     T[e] = make_double2(sh.B[e].x * f, sh.B[e].y * f);
