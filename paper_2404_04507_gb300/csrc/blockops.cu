@@ -493,14 +493,17 @@ iwf_status gram(const Batch& bt, const BlockList& A, const BlockList& B, long lo
   if (sizeof(T) == 8 && bt.engine == kEngineTensor)
     return gram_tc(bt, A, B, N, out, reinterpret_cast<double*>(partial), slots_per_prob, bt.err, s,
                    herm);
+  const bool df = sizeof(T) == 8 && bt.engine == kEngineDF;
   // at least eight tiles a CTA where that still gives every SM one (a partial of up to 83 KB for
-  // each 16-row tile cost more than the tile)
+  // each 16-row tile cost more than the tile); in FP64 the tile costs more, and as many CTAs as
+  // there are slots even out the last wave (20736 rows, 72 x 72: 932 us in 162 CTAs, 560 in 608)
   const long long tiles = (N + kGramRows - 1) / kGramRows;
-  const long long want = std::max<long long>((152 + bt.nprob - 1) / bt.nprob, tiles / 8);
+  const long long want = sizeof(T) == 8 && !df
+                             ? tiles
+                             : std::max<long long>((152 + bt.nprob - 1) / bt.nprob, tiles / 8);
   const int g = (int)std::min<long long>(std::min<long long>(tiles, want), slots_per_prob);
   const int U = (ma + kGramTx - 1) / kGramTx, V = (mb + kGramTx - 1) / kGramTx;
   const dim3 grid(g, bt.nprob);
-  const bool df = sizeof(T) == 8 && bt.engine == kEngineDF;
   switch (U * 4 + V + (herm ? 100 : 0)) {
 #define IWF_GRAM(U_, V_, H_) \
     case U_ * 4 + V_ + (H_ ? 100 : 0): \
