@@ -87,8 +87,9 @@ __device__ void householder_chain(SmallShared& sh, int n, int i) {
   const double2 al = col[0];
   const double a2 = fma(al.x, al.x, al.y * al.y);
   // above about 1e-290 (compared as integers: an FP64 comparison costs as much as a product);
-  // a NaN goes on
-  const bool reflect = __double2hiint(s2) > 0x03000000, has_al = __double2hiint(a2) > 0x03000000;
+  // a NaN, of either sign, goes on
+  const auto nonzero = [](double v) { return (__double2hiint(v) & 0x7fffffff) > 0x03000000; };
+  const bool reflect = nonzero(s2), has_al = nonzero(a2);
   const double tot = s2 + a2;
   // lane 1: 1 / |alpha|, the others 1 / |x|
   const double q = lane == 1 ? (has_al ? a2 : 1.0) : (reflect || has_al ? tot : 1.0);

@@ -114,3 +114,16 @@ def test_nearly_dependent_blocks(kind, b):
     Q = Y[:, mask == 1]
     assert np.max(np.abs(Q.conj().T @ Q - np.eye(Q.shape[1]))) <= 1e-14
     assert np.max(np.abs(X.conj().T @ Q)) <= 2.0 ** -53 * 1e7
+
+
+@pytest.mark.parametrize("bits", [0xFFF8000000000000, 0x7FF8000000000000])
+@pytest.mark.parametrize("row,col", [(5, 0), (7, 6), (40, 21), (71, 70)])
+def test_a_nan_off_the_diagonal_reaches_every_eigenvalue(row, col, bits):
+    # a quiet NaN with the sign that the GPU's own arithmetic gives it, and with the other one
+    rng = np.random.default_rng(2)
+    A = _randn(rng, 72, 72)
+    A = A + A.conj().T
+    nan = np.array([bits], dtype=np.uint64).view(np.float64)[0]
+    A[row, col], A[col, row] = complex(nan, nan), complex(nan, -nan)
+    theta, Cx, _, _, _ = rayleigh_ritz(A, 24, 24)
+    assert np.all(np.isnan(theta)) and np.all(np.isnan(Cx))
