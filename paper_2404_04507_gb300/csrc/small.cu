@@ -10,9 +10,9 @@
 //     chains that do not depend on one another on different quarters of the SM;
 //   - bisection, which needs no last bit, counts eigenvalues in double-float arithmetic on the
 //     FP32 pipes (5x the FP64 rate); inverse iteration and Rayleigh quotients are FP64.
-// Measured on one GB300, Rayleigh-Ritz with 72 basis vectors and 24 pairs: 1.14 ms (reduction 0.50,
-// bisection 0.06, inverse iteration 0.11, back-transformation 0.24, P coefficients 0.23), m = 12
-// with 4 pairs 0.10 ms. Cyclic Jacobi in double-float arithmetic, which this replaced, took 6.2
+// Measured on one GB300, Rayleigh-Ritz with 72 basis vectors and 24 pairs: 1.24 ms (reduction 0.50,
+// bisection 0.06, inverse iteration 0.11, back-transformation 0.24, P coefficients 0.33), m = 12
+// with 4 pairs 0.11 ms. Cyclic Jacobi in double-float arithmetic, which this replaced, took 6.2
 // and 0.30 ms (8 to 13 sweeps of 71 rounds at about 19k cycles) and left residuals near 1e-10 on
 // matrices with entries near 10^3; errors are now those of FP64 (residuals 2e-16 |A|).
 #include <algorithm>
@@ -778,116 +778,88 @@ __device__ void small_multiply(const double2* Y, const double2* T, double2* Z, i
   __syncthreads();
 }
 
-// Complex double-float: a double2's 16 bytes.
-struct CDF { DF re, im; };
-__device__ __forceinline__ CDF cdf_of(double2 v) {
-  CDF o;
-  split_bits(v.x, o.re.h, o.re.l);
-  split_bits(v.y, o.im.h, o.im.l);
-  return o;
-}
-// s += a b (ai_sign 1) or conj(a) b (-1)
-__device__ __forceinline__ void cdf_mac(CDF& s, CDF a, CDF b, float ai_sign) {
-  df_mac(s.re.h, s.re.l, a.re.h, a.re.l, b.re.h, b.re.l);
-  df_mac(s.re.h, s.re.l, -ai_sign * a.im.h, -ai_sign * a.im.l, b.im.h, b.im.l);
-  df_mac(s.im.h, s.im.l, a.re.h, a.re.l, b.im.h, b.im.l);
-  df_mac(s.im.h, s.im.l, ai_sign * a.im.h, ai_sign * a.im.l, b.re.h, b.re.l);
-}
-__device__ __forceinline__ DF df_mul(DF a, DF b) {
-  DF o{0.f, 0.f};
-  df_mac(o.h, o.l, a.h, a.l, b.h, b.l);
-  return df_norm(o.h, o.l);
-}
-__device__ __forceinline__ DF df_rsqrt(DF a) {        // one Newton step from the FP32 value
-  const float r = rsqrtf(a.h);
-  const DF rr = df_mul(DF{r, 0.f}, DF{r, 0.f}), p = df_mul(a, rr);
-  return df_norm(r, 0.5f * r * ((1.f - p.h) - p.l));
-}
-__device__ __forceinline__ CDF cdf_scale(CDF a, DF f) { return CDF{df_mul(a.re, f), df_mul(a.im, f)}; }
-// sum of a value over the warp, in every lane
-__device__ __forceinline__ CDF cdf_warp_sum(CDF s) {
+// Sum over the warp, in every lane.
+__device__ __forceinline__ double2 warp_sum(double2 s) {
   for (int o = 16; o; o >>= 1) {
-    float h, e;
-    two_sum(s.re.h, __shfl_xor_sync(0xffffffffu, s.re.h, o), h, e);
-    s.re = df_norm(h, e + (s.re.l + __shfl_xor_sync(0xffffffffu, s.re.l, o)));
-    two_sum(s.im.h, __shfl_xor_sync(0xffffffffu, s.im.h, o), h, e);
-    s.im = df_norm(h, e + (s.im.l + __shfl_xor_sync(0xffffffffu, s.im.l, o)));
+    s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+    s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
   }
   return s;
 }
 
-// First round of the P coefficients, in double-float arithmetic: Y = the columns in sh.B (m x b,
-// rows below x_rows zero) minus their projection on the orthonormal X in sh.A, scaled to unit norm
-// and orthonormalised by modified Gram-Schmidt; back to sh.B. Columns of norm up to 1e-12, and
-// columns within 1e-7 of the span of those before them, become zero with sh.keep 0.
+// First round of the P coefficients: Y = the columns in sh.B (m x b, rows below x_rows zero) minus
+// their projection on the orthonormal X in sh.A, scaled to unit norm and orthonormalised by
+// modified Gram-Schmidt; back to sh.B. Columns of norm up to 1e-12, and columns within 1e-7 of the
+// span of those before them, become zero with sh.keep 0. In FP64: double-float arithmetic took
+// 130 us less at 72 x 24, but left the span 1e-14 to 1e-13 off (now 4e-16).
 __device__ void p_columns_near(SmallShared& sh, int m, int b, int x_rows) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int kWarps = kSmallThreads / 32;
   const int ld = m | 1;                                // column-major, odd stride: no conflicts
-  CDF* X = reinterpret_cast<CDF*>(sh.V);
-  CDF* Y = X + kMaxBlock * (kMaxSmall + 1);
-  CDF* G = Y + kMaxBlock * (kMaxSmall + 1);
+  double2* X = sh.V;
+  double2* Y = X + kMaxBlock * (kMaxSmall + 1);
+  double2* G = Y + kMaxBlock * (kMaxSmall + 1);
   static_assert(2 * kMaxBlock * (kMaxSmall + 1) + kMaxBlock * kMaxBlock <= kMaxSmall * kMaxSmall, "work");
   for (int e = tid; e < m * b; e += kSmallThreads) {
     const int i = e / b, c = e - i * b;
-    X[c * ld + i] = cdf_of(sh.A[e]);
-    Y[c * ld + i] = cdf_of(sh.B[e]);
+    X[c * ld + i] = sh.A[e];
+    Y[c * ld + i] = sh.B[e];
   }
   __syncthreads();
   // G = X^H Y: Hermitian, since Y is X with rows zeroed
   for (int e = tid; e < b * (b + 1) / 2; e += kSmallThreads) {
     int r, c;
     fold(e, b, r, c);
-    CDF s{};
-    for (int i = x_rows; i < m; ++i) cdf_mac(s, X[r * ld + i], Y[c * ld + i], -1.f);
+    double2 s = make_double2(0.0, 0.0);
+    for (int i = x_rows; i < m; ++i) s = cmac_conj(X[r * ld + i], Y[c * ld + i], s);
+    if (r == c) s.y = 0.0;
     G[r * b + c] = s;
-    G[c * b + r] = CDF{s.re, DF{-s.im.h, -s.im.l}};
+    G[c * b + r] = make_double2(s.x, -s.y);
   }
   __syncthreads();
   for (int e = tid; e < m * b; e += kSmallThreads) {
     const int c = e / m, i = e - c * m;
-    CDF s = Y[c * ld + i];
+    double2 s = Y[c * ld + i];
     for (int r = 0; r < b; ++r) {
-      const CDF g = G[r * b + c];
-      cdf_mac(s, X[r * ld + i], CDF{DF{-g.re.h, -g.re.l}, DF{-g.im.h, -g.im.l}}, 1.f);
+      const double2 g = G[r * b + c];
+      s = cmac(X[r * ld + i], make_double2(-g.x, -g.y), s);
     }
     Y[c * ld + i] = s;
   }
   __syncthreads();
+  const auto dot = [&](const double2* a, const double2* y) {   // a^H y, in every lane
+    double2 s = make_double2(0.0, 0.0);
+    for (int i = lane; i < m; i += 32) s = cmac_conj(a[i], y[i], s);
+    return warp_sum(s);
+  };
   for (int c = warp; c < b; c += kWarps) {             // unit columns
-    CDF s{};
-    for (int i = lane; i < m; i += 32) cdf_mac(s, Y[c * ld + i], Y[c * ld + i], -1.f);
-    s = cdf_warp_sum(s);
-    const bool on = s.re.h > 1e-24f;
-    const DF f = on ? df_rsqrt(s.re) : DF{0.f, 0.f};
-    for (int i = lane; i < m; i += 32) Y[c * ld + i] = cdf_scale(Y[c * ld + i], f);
+    const double n2 = dot(Y + c * ld, Y + c * ld).x;
+    const double f = n2 > 1e-24 ? rsqrt(n2) : 0.0;
+    for (int i = lane; i < m; i += 32) Y[c * ld + i] = make_double2(Y[c * ld + i].x * f, Y[c * ld + i].y * f);
   }
   __syncthreads();
   for (int l = 0; l < b; ++l) {
+    const double2* yl = Y + l * ld;
     for (int j = l + warp; j < b; j += kWarps) {
-      CDF s{};
-      for (int i = lane; i < m; i += 32) cdf_mac(s, Y[l * ld + i], Y[j * ld + i], -1.f);
-      s = cdf_warp_sum(s);
+      const double2 s = dot(yl, Y + j * ld);
       if (lane == 0) G[j] = s;
     }
     __syncthreads();
-    const CDF n2 = G[l];
-    const bool on = n2.re.h > 1e-14f;
-    const DF f = on ? df_rsqrt(n2.re) : DF{0.f, 0.f};
-    const DF f2 = df_mul(f, f);
+    const double n2 = G[l].x;
+    const bool on = n2 > 1e-14;
+    const double f = on ? rsqrt(n2) : 0.0, f2 = f * f;
     for (int j = l + 1 + warp; on && j < b; j += kWarps) {
-      const CDF g = cdf_scale(G[j], DF{-f2.h, -f2.l});
-      for (int i = lane; i < m; i += 32) cdf_mac(Y[j * ld + i], Y[l * ld + i], g, 1.f);
+      const double2 g = make_double2(-G[j].x * f2, -G[j].y * f2);
+      for (int i = lane; i < m; i += 32) Y[j * ld + i] = cmac(yl[i], g, Y[j * ld + i]);
     }
     __syncthreads();
-    for (int i = tid; i < m; i += kSmallThreads) Y[l * ld + i] = cdf_scale(Y[l * ld + i], f);
+    for (int i = tid; i < m; i += kSmallThreads) Y[l * ld + i] = make_double2(yl[i].x * f, yl[i].y * f);
     if (tid == 0) sh.keep[l] = on;
   }
   __syncthreads();
   for (int e = tid; e < m * b; e += kSmallThreads) {
     const int i = e / b, c = e - i * b;
-    const CDF y = Y[c * ld + i];
-    sh.B[e] = make_double2((double)y.re.h + (double)y.re.l, (double)y.im.h + (double)y.im.l);
+    sh.B[e] = Y[c * ld + i];
   }
   __syncthreads();
 }
@@ -948,11 +920,11 @@ rr_kernel(Batch bt, const double2* Ain, int m, int b, const int* mask, int x_row
     sh.B[e] = (e / b) < x_rows ? make_double2(0, 0) : c;
   }
   __syncthreads();
-  // Cp in two rounds of (orthogonalise against Cx, then orthonormalise). The first only has to
-  // come near: it runs in double-float arithmetic, columns scaled to unit norm (down to 1e-12)
-  // and orthonormalised by Gram-Schmidt. The second removes in FP64 what normalising tiny columns
-  // left of Cx in them, and restores orthonormality to FP64 rounding: one projection, one Gram
-  // matrix and, since the columns are orthonormal to better than 1e-6, a series.
+  // Cp in two rounds of (orthogonalise against Cx, then orthonormalise). The first scales the
+  // columns to unit norm (down to 1e-12) and orthonormalises them by Gram-Schmidt. The second
+  // removes what normalising tiny columns left of Cx in them, and restores orthonormality to
+  // rounding: one projection, one Gram matrix and, since the columns are orthonormal to better than
+  // 1e-6, a series.
   p_columns_near(sh, m, b, x_rows);
   double2* X = sh.A;
   double2 *M = sh.A + kLu, *T = M + kMaxBlock * kMaxBlock;

@@ -127,3 +127,38 @@ def test_a_nan_off_the_diagonal_reaches_every_eigenvalue(row, col, bits):
     A[row, col], A[col, row] = complex(nan, nan), complex(nan, -nan)
     theta, Cx, _, _, _ = rayleigh_ritz(A, 24, 24)
     assert np.all(np.isnan(theta)) and np.all(np.isnan(Cx))
+
+
+def _orthonormal(Y):
+    """An orthonormal basis of Y's columns in extended precision."""
+    Q = []
+    for v in Y.T:
+        for _ in range(3):
+            for q in Q:
+                v = v - q * np.vdot(q, v)
+        Q.append(v / np.sqrt(np.vdot(v, v).real))
+    return np.stack(Q, 1)
+
+
+@pytest.mark.parametrize("coupling", [1.0, 1e-3, 1e-8])
+@pytest.mark.parametrize("m,b", [(72, 24), (36, 12), (9, 3)])
+def test_p_coefficients_span_what_they_should(m, b, coupling):
+    # S Cp spans the W and P parts of Cx's columns, orthogonal to S Cx. A column of it comes from a sum
+    # of b + 2 products of unit columns, (b + 2) 2^-53 at worst before the orthonormalisation, whose
+    # condition (below 20 here) multiplies rms errors a fifth of that: 64 2^-53 bounds the part
+    # outside the exact span
+    rng = np.random.default_rng(m)
+    R = _randn(rng, m, m) * coupling
+    A = np.diag(np.sort(rng.uniform(1.0, 100.0, m))) + R + R.conj().T
+    theta, Cx, Cp, mask_p, status = rayleigh_ritz(A, b, b)
+    assert status == 0 and np.all(mask_p == 1)
+    assert np.max(np.abs(theta - np.linalg.eigvalsh(A)[:b])) <= 1e-14 * np.linalg.norm(A, 2)
+    for U, V, eye in ((Cx, Cx, np.eye(b)), (Cp, Cp, np.eye(b)), (Cx, Cp, 0.0)):
+        assert np.max(np.abs(U.conj().T @ V - eye)) <= 1e-14
+    X = _orthonormal(Cx.astype(np.clongdouble))
+    Y = Cx.astype(np.clongdouble)
+    Y[:b] = 0
+    Y = Y - X @ (X.conj().T @ Y)
+    Q = _orthonormal(Y / np.sqrt(np.sum(np.abs(Y) ** 2, axis=0)))
+    out = Cp - Q @ (Q.conj().T @ Cp)
+    assert np.max(np.sqrt(np.sum(np.abs(out) ** 2, axis=0))) <= 64 * 2.0 ** -53
