@@ -446,24 +446,28 @@ iwf_status scratch_pool(cudaMemPool_t* out) {
   return IWF_OK;
 }
 
+// One allocation a call: each costs the host several us with its release (two made a small
+// iwf_block_update 62 us where cudaMalloc and cudaFree had made it 45; one, 42).
 struct Scratch {
   cudaStream_t st;
-  std::vector<void*> ptrs;
+  char* base = nullptr;
   explicit Scratch(cudaStream_t s) : st(s) {}
-  ~Scratch() { for (void* p : ptrs) cudaFreeAsync(p, st); }
-  iwf_status get(void** out, size_t bytes) {
+  ~Scratch() { if (base) cudaFreeAsync(base, st); }
+  iwf_status get(size_t bytes) {
     cudaMemPool_t pool;
     IWF_TRY(scratch_pool(&pool));
-    if (cudaMallocFromPoolAsync(out, bytes, pool, st) != cudaSuccess) {
+    if (cudaMallocFromPoolAsync((void**)&base, bytes, pool, st) != cudaSuccess) {
       (void)cudaGetLastError();
+      base = nullptr;
       return iwf::fail(IWF_ERR_ALLOC, "contraction scratch");
     }
-    ptrs.push_back(*out);
     return IWF_OK;
   }
 };
 
-iwf_status contract_batch(int engine, Scratch& sc, iwf::Batch* bt) {
+// The call's scratch: column scales, error word, then `bytes` more (from *more on).
+constexpr size_t kContractHead = (sizeof(int) * (2 * iwf::kMaxSmall + 1) + 255) / 256 * 256;
+iwf_status contract_batch(int engine, Scratch& sc, iwf::Batch* bt, size_t bytes, void** more) {
   if (engine != IWF_CONTRACT_TENSOR && engine != IWF_CONTRACT_DF && engine != IWF_CONTRACT_F64)
     return iwf::fail(IWF_ERR_ARG, "unknown contraction engine");
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;   // the call synchronises
@@ -476,12 +480,11 @@ iwf_status contract_batch(int engine, Scratch& sc, iwf::Batch* bt) {
   bt->engine = engine == IWF_CONTRACT_TENSOR ? iwf::kEngineTensor
                : engine == IWF_CONTRACT_DF   ? iwf::kEngineDF
                                              : iwf::kEngineF64;
-  void *e = nullptr, *w = nullptr;
-  IWF_TRY(sc.get(&e, sizeof(int) * 2 * iwf::kMaxSmall));
-  IWF_TRY(sc.get(&w, sizeof(int)));
-  IWF_CUDA(cudaMemsetAsync(w, 0, sizeof(int), sc.st));
-  bt->exps = static_cast<int*>(e);
-  bt->err = static_cast<int*>(w);
+  IWF_TRY(sc.get(kContractHead + bytes));
+  bt->exps = reinterpret_cast<int*>(sc.base);
+  bt->err = bt->exps + 2 * iwf::kMaxSmall;
+  if (more) *more = sc.base + kContractHead;
+  IWF_CUDA(cudaMemsetAsync(bt->err, 0, sizeof(int), sc.st));
   return IWF_OK;
 }
 
@@ -505,17 +508,15 @@ iwf_status iwf_gram(int engine, long long nrows, const void* A, int ma, const vo
   cudaStream_t st = (cudaStream_t)stream;
   Scratch sc(st);
   Batch bt;
-  IWF_TRY(contract_batch(engine, sc, &bt));
   // the tensor engine has one slot per SM and sub-Gram of 48 x 24 columns at most (5.6 MB)
   const int slots = engine == IWF_CONTRACT_TENSOR ? 76 : 608;
-  void *part = nullptr, *out = nullptr;
-  IWF_TRY(sc.get(&part, sizeof(double2) * (size_t)slots * kCapG));
-  IWF_TRY(sc.get(&out, sizeof(double2) * kCapG));
+  void* more = nullptr;
+  IWF_TRY(contract_batch(engine, sc, &bt, sizeof(double2) * kCapG * ((size_t)slots + 1), &more));
+  double2 *out = static_cast<double2*>(more), *part = out + kCapG;
   BlockList LA{}, LB{};
   LA.p[0] = A; LA.nb = 1; LA.b = ma;
   LB.p[0] = B; LB.nb = 1; LB.b = mb;
-  IWF_TRY(gram<double>(bt, LA, LB, nrows, static_cast<double2*>(out),
-                       static_cast<double2*>(part), slots, st, false));
+  IWF_TRY(gram<double>(bt, LA, LB, nrows, out, part, slots, st, false));
   IWF_CUDA(cudaMemcpyAsync(G, out, sizeof(double2) * (size_t)ma * mb, cudaMemcpyDeviceToDevice, st));
   return contract_finish(bt, st);
 }
@@ -529,7 +530,7 @@ iwf_status iwf_block_update(int engine, long long nrows, const void* S, int m, c
   cudaStream_t st = (cudaStream_t)stream;
   Scratch sc(st);
   Batch bt;
-  IWF_TRY(contract_batch(engine, sc, &bt));
+  IWF_TRY(contract_batch(engine, sc, &bt, 0, nullptr));
   BlockList LS{};
   LS.p[0] = S; LS.nb = 1; LS.b = m;
   IWF_TRY(block_update<double>(bt, LS, nrows, static_cast<const double2*>(C), nullptr, m * q, q,
