@@ -262,11 +262,15 @@ iwf_status launch_direct(DirectArgs a, bool real, int nprob, cudaStream_t s) {
   // A slice is shared among CTAs where there are fewer than four an SM: a window of few slices
   // (8^4 x 16, 48 real modes, 4 vectors: 16 CTAs, 390 us where the transforms take 164) otherwise
   // leaves the chip idle (now 45 us). With four or more, sharing only repeats the shifts' set-up.
-  int sms = 0, dev = 0;
-  IWF_CUDA(cudaGetDevice(&dev));
-  IWF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const long long want = 4LL * sms / std::max(1LL, slices * nprob * a.groups);
-  a.parts = (int)std::max(1LL, std::min<long long>(want, (a.g.MI + a.P - 1) / a.P));
+  const long long rounds = (a.g.MI + a.P - 1) / a.P;
+  a.parts = 1;
+  if (rounds > 1) {
+    int sms = 0, dev = 0;
+    IWF_CUDA(cudaGetDevice(&dev));
+    IWF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const long long want = 4LL * sms / std::max(1LL, slices * nprob * a.groups);
+    a.parts = (int)std::max(1LL, std::min(want, rounds));
+  }
   const long long blocks = slices * a.parts;
   if ((long long)nprob * a.groups > 65535 || blocks > 2147483647LL)
     return fail(IWF_ERR_UNSUPPORTED, "direct apply: too many slices or vectors");
