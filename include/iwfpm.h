@@ -440,7 +440,8 @@ iwf_status iwf_apply_stencil(iwf_plan* plan, int precision, const void* psi, voi
  *                    global memory directly, with one shared-memory transpose per pass;
  *                    needs n = 4, d = 2 with 2K_1 = 2K_2 and 2L_1 = 2L_2, each 16 or 32;
  *   IWF_PATH_AUTO    the direct convolution for potentials with few modes (iwf_apply); else
- *                    the pencil path where the geometry allows it, else the tiled path.
+ *                    the path the autotuner kept, or without it the pencil path where the
+ *                    geometry allows it, else the tiled path.
  */
 enum { IWF_PATH_AUTO = 0, IWF_PATH_TILED = 1, IWF_PATH_PENCIL = 2 };
 
@@ -450,12 +451,13 @@ enum { IWF_PATH_AUTO = 0, IWF_PATH_TILED = 1, IWF_PATH_PENCIL = 2 };
  * precision. Candidates: the tiled path with threads per CTA {128, 256}, shared-memory tile
  * budget {24, 48, 96, 160} KB and L2 chunk of vectors between passes {24, 48, 96} MB; where
  * the geometry allows it, the pencil path with chunks {12, 24, 48, 96} MB. On a plan whose path
- * is IWF_PATH_AUTO the direct convolution takes part where the potential allows it; when it
- * wins the path stays IWF_PATH_AUTO, with the best schedule of the transforms kept for other
- * potentials. Host outputs (may be NULL): *best_ms per apply, best[3] = {threads, tile_kb, chunk_mb} (threads and
- * tile_kb are 0 when the pencil path won; iwf_plan_get_schedule reports the path). Needs a
- * potential. Results are identical for every schedule up to floating-point summation order;
- * synchronises.
+ * is IWF_PATH_AUTO the direct convolution takes part where the potential allows it; unless it
+ * takes part and loses, the path stays IWF_PATH_AUTO, and the fastest transforms (kernels and
+ * schedule) are kept for potentials of more modes. Host outputs (may be NULL): *best_ms per apply
+ * of the fastest candidate, the direct convolution included; best[3] = {threads, tile_kb,
+ * chunk_mb} of the fastest transforms (threads and tile_kb are 0 for the pencil path;
+ * iwf_plan_get_schedule reports the path). Needs a potential. Results are identical for every
+ * schedule up to floating-point summation order; synchronises.
  */
 iwf_status iwf_plan_autotune(iwf_plan* plan, int precision, int nvec, double* best_ms,
                              int* best, void* stream);
@@ -486,8 +488,11 @@ iwf_status iwf_plan_set_path(iwf_plan* plan, int precision, int path);
 enum { IWF_ARITH_F64 = 0, IWF_ARITH_DF = 1 };
 iwf_status iwf_plan_set_arith(iwf_plan* plan, int arith);
 
-/* The schedule iwf_apply will use: sched[4] = {threads, tile_kb, chunk_mb, path}, path
- * being IWF_PATH_TILED or IWF_PATH_PENCIL (IWF_PATH_AUTO resolved for this geometry). */
+/* The schedule of the transforms: sched[4] = {threads, tile_kb, chunk_mb, path}, path being
+ * IWF_PATH_TILED or IWF_PATH_PENCIL (IWF_PATH_AUTO resolved for this geometry, or as autotuned).
+ * With IWF_PATH_AUTO iwf_apply uses it for the potentials it does not apply by direct
+ * convolution; whether it does is not part of a schedule (iwf_kernel_launches tells: one launch,
+ * or three and more). */
 iwf_status iwf_plan_get_schedule(const iwf_plan* plan, int precision, int* sched);
 
 /* Number of kernels this library has launched in this process (all devices, all plans). */

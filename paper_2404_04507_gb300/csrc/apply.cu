@@ -1094,6 +1094,14 @@ bool pencil_geometry(const Geom& g, int* LI, int* LII) {
   return true;
 }
 
+// The kernel set of a plan's transforms: the path set, or with IWF_PATH_AUTO the one the autotuner
+// kept, or else the pencil set where the geometry allows it.
+int transforms_path(const iwf_plan* p, int ti) {
+  int LI = 0, LII = 0;
+  const int path = p->path[ti] == IWF_PATH_AUTO ? p->auto_path[ti] : p->path[ti];
+  return path != IWF_PATH_TILED && pencil_geometry(p->g, &LI, &LII) ? IWF_PATH_PENCIL : IWF_PATH_TILED;
+}
+
 // Threads of a pass A/C CTA and tile columns of a pass B CTA: 64 KB of shared memory each.
 template <typename T> constexpr int pencil_threads() { return sizeof(T) == 4 ? 256 : 128; }
 
@@ -1345,7 +1353,7 @@ iwf_status apply_typed(iwf_plan* p, const void* psi, void* hpsi, int nvec, cudaS
   Cp.lam = sizeof(T) == 8 ? (const void*)p->d_lam64 : (const void*)p->d_lam32;
 
   int LI = 0, LII = 0;
-  if (p->path[ti] != IWF_PATH_TILED && pencil_geometry(g, &LI, &LII)) {
+  if (transforms_path(p, ti) == IWF_PATH_PENCIL && pencil_geometry(g, &LI, &LII)) {
     // pencil geometry: N = LI^2 LII^2 <= 2^20, so in-vector offsets fit in int
     PencilArgs pa{};
     pa.lo = p->d_lo; pa.pot = pot; pa.ld = g.N; pa.MI = g.MI; pa.MII = g.MII;
@@ -1487,15 +1495,17 @@ iwf_status autotune_impl(iwf_plan* p, int precision, int nvec, double* best_ms, 
                       (ti == 0 ? direct_pays<double>(p, nullptr) : direct_pays<float>(p, nullptr));
   if (direct) trial(IWF_PATH_AUTO, bt, bk, bc);
   p->tune_threads[ti] = bt; p->tune_tile_kb[ti] = bk; p->tune_chunk_mb[ti] = bc;
-  const int natural = pencil_geometry(p->g, &LI, &LII) ? IWF_PATH_PENCIL : IWF_PATH_TILED;
-  p->path[ti] = saved_path == IWF_PATH_AUTO && (direct ? direct_t < best_t : bp == natural)
-                    ? IWF_PATH_AUTO : bp;
+  const bool keep_auto = saved_path == IWF_PATH_AUTO && (!direct || direct_t < best_t);
+  if (st == IWF_OK) {
+    p->path[ti] = keep_auto ? IWF_PATH_AUTO : bp;
+    p->auto_path[ti] = keep_auto ? bp : IWF_PATH_AUTO;
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   cudaFree(x);
   cudaFree(y);
   if (st != IWF_OK) { p->path[ti] = saved_path; return st; }
-  if (best_ms) *best_ms = p->path[ti] == IWF_PATH_AUTO ? std::fmin(best_t, direct_t) : best_t;
+  if (best_ms) *best_ms = std::fmin(best_t, direct_t);
   if (best) {
     best[0] = bp == IWF_PATH_PENCIL ? 0 : bt;
     best[1] = bp == IWF_PATH_PENCIL ? 0 : bk;
@@ -1559,7 +1569,9 @@ iwf_status set_path_impl(iwf_plan* p, int precision, int path) {
   if (path == IWF_PATH_TILED && precision == IWF_PREC_F64 && p->fft_arith == IWF_ARITH_DF)
     return fail(IWF_ERR_UNSUPPORTED,
                 "iwf_plan_set_path: double-float DFTs are set on this plan and need the pencil path");
-  p->path[precision == IWF_PREC_F64 ? 0 : 1] = path;
+  const int ti = precision == IWF_PREC_F64 ? 0 : 1;
+  p->path[ti] = path;
+  p->auto_path[ti] = IWF_PATH_AUTO;
   return IWF_OK;
 }
 
@@ -1567,7 +1579,7 @@ iwf_status set_arith_impl(iwf_plan* p, int arith) {
   if (arith != IWF_ARITH_F64 && arith != IWF_ARITH_DF)
     return fail(IWF_ERR_ARG, "iwf_plan_set_arith: unknown arithmetic");
   int LI = 0, LII = 0;
-  if (arith == IWF_ARITH_DF && (!pencil_geometry(p->g, &LI, &LII) || p->path[0] == IWF_PATH_TILED))
+  if (arith == IWF_ARITH_DF && (!pencil_geometry(p->g, &LI, &LII) || transforms_path(p, 0) == IWF_PATH_TILED))
     return fail(IWF_ERR_UNSUPPORTED,
                 "iwf_plan_set_arith: double-float DFTs need the pencil path (n = 4, d = 2, two "
                 "equal axis lengths per group, each 16 or 32)");
@@ -1580,12 +1592,10 @@ iwf_status get_schedule_impl(const iwf_plan* p, int precision, int* sched) {
     return fail(IWF_ERR_ARG, "iwf_plan_get_schedule: unknown precision");
   if (!sched) return fail(IWF_ERR_ARG, "iwf_plan_get_schedule: NULL output");
   const int ti = precision == IWF_PREC_F64 ? 0 : 1;
-  int LI = 0, LII = 0;
-  const bool pencil = p->path[ti] != IWF_PATH_TILED && pencil_geometry(p->g, &LI, &LII);
   sched[0] = p->tune_threads[ti];
   sched[1] = p->tune_tile_kb[ti];
   sched[2] = p->tune_chunk_mb[ti];
-  sched[3] = pencil ? IWF_PATH_PENCIL : IWF_PATH_TILED;
+  sched[3] = transforms_path(p, ti);
   return IWF_OK;
 }
 

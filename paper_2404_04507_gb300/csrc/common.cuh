@@ -186,6 +186,8 @@ struct iwf_plan {
   // apply kernels per precision: IWF_PATH_AUTO (pencil path where the geometry allows it),
   // IWF_PATH_TILED or IWF_PATH_PENCIL
   int path[2] = {IWF_PATH_AUTO, IWF_PATH_AUTO};
+  // the transforms IWF_PATH_AUTO falls back on: as autotuned, or by the geometry (IWF_PATH_AUTO)
+  int auto_path[2] = {IWF_PATH_AUTO, IWF_PATH_AUTO};
   // DFT arithmetic of FP64 applies on the pencil path (IWF_ARITH_F64 or IWF_ARITH_DF)
   int fft_arith = IWF_ARITH_F64;
   // eigensolver workspace of iwf_eigensolve / iwf_batch_eigensolve, kept between solves: the

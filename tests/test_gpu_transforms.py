@@ -190,3 +190,33 @@ def test_host_blocks(iwf):  # noqa: F811
             plan.set_path(prec, path)
             x = torch.from_numpy(np.ascontiguousarray(_block(plan, 7, prec, 8).T)).to(DTYPE[prec])
             assert torch.equal(plan.apply_host(x), plan.apply(x.cuda()).cpu())
+
+
+@pytest.mark.parametrize("prec", ["f64", "c64"])
+@pytest.mark.parametrize("K,L,nvec", [(8, 8, 1), (8, 8, 16), (8, 16, 2), (16, 8, 1)])
+def test_autotune_keeps_the_transforms_it_reports(iwf, prec, K, L, nvec):  # noqa: F811
+    # tuned with a potential that the direct convolution applies; a later one of many modes runs on
+    # the kernels of the best schedule, bit for bit those of the path that the plan reports
+    pb = W.config_moire(eps=0.5, K=K, L=L)
+    plan = _plan(iwf, pb)
+    ms, best = plan.autotune(prec, nvec=nvec)
+    sched = plan.schedule(prec)
+    assert ms > 0 and (sched["path"] == "pencil") == (best[:2] == (0, 0))
+    plan.set_potential(*W.random_modes(4, 30, 3, seed=9))
+    x = torch.from_numpy(np.ascontiguousarray(_block(plan, nvec, prec, 3).T)).to(DTYPE[prec]).cuda()
+    got = plan.apply(x)
+    plan.set_path(prec, sched["path"])
+    assert torch.equal(got, plan.apply(x))
+    plan.set_path(prec, "auto")
+    assert plan.schedule(prec)["path"] == "pencil"
+
+
+def test_a_tuned_tiled_path_refuses_double_float_dfts(iwf):  # noqa: F811
+    from paper_2404_04507_gb300 import capi
+    pb = PENCIL["moire16"]
+    plan = _plan(iwf, pb)
+    plan.set_path("f64", "tiled")
+    plan.autotune("f64", nvec=1)
+    with pytest.raises(capi.IwfError) as e:
+        plan.set_arith("df")
+    assert e.value.status == -10
