@@ -126,6 +126,8 @@ struct ApplyBatch {
 
 }  // namespace iwf
 
+constexpr int kNoStencil = 1 << 30;        // more modes than any direct apply takes
+
 struct iwf_plan {
   int device = 0;
   int method = IWF_METHOD_IWFPM;
@@ -152,7 +154,7 @@ struct iwf_plan {
   int tab_off[IWF_MAX_N] = {};
   // folded modes of the potential for the direct-convolution apply, without the constant term
   // (vconst): stencil_m[q*n + j] in [0, lens[j]), coefficient stencil_c[q] = Vg (re, im)
-  int stencil_nm = 0;
+  int stencil_nm = 0;                     // kNoStencil: the upload failed, no direct apply
   bool stencil_const = false;             // the potential has a constant term
   bool stencil_real = false;              // every coefficient is real
   int* d_stencil_m = nullptr;

@@ -366,7 +366,7 @@ iwf_status build_potential(iwf_plan* p, int nmodes, const int* m, const double* 
   cudaFree(p->d_stencil_c);
   p->d_stencil_m = nullptr;
   p->d_stencil_c = nullptr;
-  p->stencil_nm = 0;
+  p->stencil_nm = kNoStencil;              // until they are on the device: an apply takes the tables
   direct_modes(F, n, p->h_stencil_m, p->h_stencil_c);
   p->stencil_const = p->h_stencil_c.size() < nm;
   p->stencil_real = true;
