@@ -561,8 +561,8 @@ iwf_status iwf_plan_set_wait_limit(iwf_plan* plan, long long rounds);
  * Matrices: A (nrows x ma), B (nrows x mb), S (nrows x m) and Y (nrows x q) are device,
  * complex double, column-major with leading dimension nrows; G (ma x mb) and C (m x q) are
  * device, complex double, row-major. ma, mb, m <= 72, q <= 24, nrows >= 1.
- * Scratch (a few MB) comes from a stream-ordered pool that keeps at most 16 MB; each call
- * synchronises `stream`.
+ * iwf_gram's partial sums (a few MB; up to 50 MB in the double-float and FP64 engines) come from a
+ * stream-ordered pool that keeps at most 32 MB; each call synchronises `stream`.
  * Errors: IWF_ERR_ARG (shape, NULL), IWF_ERR_ALLOC, IWF_ERR_CUDA, IWF_ERR_TIMEOUT (a bounded
  * wait of the tensor-core pipeline ran out).
  */

@@ -1,4 +1,5 @@
 // C-ABI entry points: plan life cycle, window export, potential, apply, preconditioner.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -420,10 +421,12 @@ iwf_status iwf_preconditioner(const iwf_plan* p, double* M, double* sigma) {
 
 // ---- the eigensolver's contractions as entry points (iwf_gram, iwf_block_update) ----------
 namespace {
-// Scratch of one call, ordered on its stream, from a pool of the library's own (one per device)
-// that keeps at most kPoolKeep bytes between calls: cudaMalloc and cudaFree of it took 0.5 ms of a
-// 2.8 ms call. The driver makes the pool safe for concurrent threads and streams.
-constexpr unsigned long long kPoolKeep = 16ull << 20;
+// Partial sums of one call, ordered on its stream, from a pool of the library's own (one per device)
+// that keeps at most kPoolKeep bytes between calls: cudaMalloc and cudaFree of them took 0.5 ms of a
+// 2.8 ms call. The driver makes the pool safe for concurrent threads and streams. The pool grows
+// by 32 MB at a time, and a limit below that kept nothing over a synchronisation (94 us a call to
+// map the memory again, 11 with it kept).
+constexpr unsigned long long kPoolKeep = 32ull << 20;
 iwf_status scratch_pool(cudaMemPool_t* out) {
   static std::mutex mu;
   static cudaMemPool_t pools[64] = {};
@@ -446,27 +449,62 @@ iwf_status scratch_pool(cudaMemPool_t* out) {
   return IWF_OK;
 }
 
-// One allocation a call: each costs the host several us with its release (two made a small
-// iwf_block_update 62 us where cudaMalloc and cudaFree had made it 45; one, 42).
+// Column scales and error word of a call: one of a few fixed places per device, held by one call
+// at a time, so that a call without partial sums (iwf_block_update) allocates nothing. From the
+// pool it took 50 to 62 us on 1000 rows where cudaMalloc and cudaFree had made it 36 to 46.
+constexpr int kContractPlaces = 64, kContractHead = 2 * iwf::kMaxSmall + 1;
+__device__ int g_contract_head[kContractPlaces][kContractHead];
+std::mutex g_head_mu;
+unsigned long long g_head_used[64] = {};               // per device, a bit a place
+int* g_head_addr[64] = {};
+
 struct Scratch {
   cudaStream_t st;
-  char* base = nullptr;
+  void* pool_mem = nullptr;
+  int dev = -1, place = -1;
+  bool done = false;                                   // the call's work is known to be complete
   explicit Scratch(cudaStream_t s) : st(s) {}
-  ~Scratch() { if (base) cudaFreeAsync(base, st); }
-  iwf_status get(size_t bytes) {
+  ~Scratch() {
+    if (place >= 0 && !done) cudaStreamSynchronize(st);
+    if (pool_mem) cudaFreeAsync(pool_mem, st);
+    if (place < 0) return;
+    std::lock_guard<std::mutex> lock(g_head_mu);
+    g_head_used[dev] &= ~(1ull << place);
+  }
+  iwf_status get(void** out, size_t bytes) {           // one block a call
     cudaMemPool_t pool;
     IWF_TRY(scratch_pool(&pool));
-    if (cudaMallocFromPoolAsync((void**)&base, bytes, pool, st) != cudaSuccess) {
+    if (cudaMallocFromPoolAsync(&pool_mem, bytes, pool, st) != cudaSuccess) {
       (void)cudaGetLastError();
-      base = nullptr;
+      pool_mem = nullptr;
       return iwf::fail(IWF_ERR_ALLOC, "contraction scratch");
     }
+    *out = pool_mem;
+    return IWF_OK;
+  }
+  // kContractHead ints; null when every place is held
+  iwf_status head(int** out) {
+    IWF_CUDA(cudaGetDevice(&dev));
+    *out = nullptr;
+    if (dev < 0 || dev >= 64) return iwf::fail(IWF_ERR_ARG, "device ordinal out of range");
+    std::lock_guard<std::mutex> lock(g_head_mu);
+    if (!g_head_addr[dev]) {
+      void* addr = nullptr;
+      IWF_CUDA(cudaGetSymbolAddress(&addr, g_contract_head));
+      g_head_addr[dev] = static_cast<int*>(addr);
+    }
+    for (int k = 0; k < kContractPlaces; ++k)
+      if (!(g_head_used[dev] >> k & 1ull)) {
+        g_head_used[dev] |= 1ull << k;
+        place = k;
+        *out = g_head_addr[dev] + (size_t)k * kContractHead;
+        return IWF_OK;
+      }
     return IWF_OK;
   }
 };
 
-// The call's scratch: column scales, error word, then `bytes` more (from *more on).
-constexpr size_t kContractHead = (sizeof(int) * (2 * iwf::kMaxSmall + 1) + 255) / 256 * 256;
+// The batch of one call; `bytes` (0: none) of scratch for its partial sums to *more.
 iwf_status contract_batch(int engine, Scratch& sc, iwf::Batch* bt, size_t bytes, void** more) {
   if (engine != IWF_CONTRACT_TENSOR && engine != IWF_CONTRACT_DF && engine != IWF_CONTRACT_F64)
     return iwf::fail(IWF_ERR_ARG, "unknown contraction engine");
@@ -480,18 +518,24 @@ iwf_status contract_batch(int engine, Scratch& sc, iwf::Batch* bt, size_t bytes,
   bt->engine = engine == IWF_CONTRACT_TENSOR ? iwf::kEngineTensor
                : engine == IWF_CONTRACT_DF   ? iwf::kEngineDF
                                              : iwf::kEngineF64;
-  IWF_TRY(sc.get(kContractHead + bytes));
-  bt->exps = reinterpret_cast<int*>(sc.base);
+  IWF_TRY(sc.head(&bt->exps));
+  const size_t extra = bt->exps ? 0 : (kContractHead * sizeof(int) + 255) / 256 * 256;
+  if (bytes + extra) {
+    void* mem = nullptr;
+    IWF_TRY(sc.get(&mem, bytes + extra));
+    if (extra) bt->exps = static_cast<int*>(mem);
+    if (more) *more = static_cast<char*>(mem) + extra;
+  }
   bt->err = bt->exps + 2 * iwf::kMaxSmall;
-  if (more) *more = sc.base + kContractHead;
   IWF_CUDA(cudaMemsetAsync(bt->err, 0, sizeof(int), sc.st));
   return IWF_OK;
 }
 
-iwf_status contract_finish(const iwf::Batch& bt, cudaStream_t st) {
+iwf_status contract_finish(const iwf::Batch& bt, Scratch& sc) {
   int h = 0;
-  IWF_CUDA(cudaMemcpyAsync(&h, bt.err, sizeof(int), cudaMemcpyDeviceToHost, st));
-  IWF_CUDA(cudaStreamSynchronize(st));
+  IWF_CUDA(cudaMemcpyAsync(&h, bt.err, sizeof(int), cudaMemcpyDeviceToHost, sc.st));
+  IWF_CUDA(cudaStreamSynchronize(sc.st));
+  sc.done = true;
   if (h) return iwf::fail(IWF_ERR_TIMEOUT, "tensor-core contraction: a bounded wait ran out");
   return IWF_OK;
 }
@@ -508,17 +552,20 @@ iwf_status iwf_gram(int engine, long long nrows, const void* A, int ma, const vo
   cudaStream_t st = (cudaStream_t)stream;
   Scratch sc(st);
   Batch bt;
-  // the tensor engine has one slot per SM and sub-Gram of 48 x 24 columns at most (5.6 MB)
-  const int slots = engine == IWF_CONTRACT_TENSOR ? 76 : 608;
+  // the tensor engine has one slot per SM and sub-Gram of 48 x 24 columns at most (5.6 MB); the
+  // others at most one per tile of 16 rows
+  const bool tensor = engine == IWF_CONTRACT_TENSOR;
+  const int slots = tensor ? 76 : (int)std::min(608LL, (nrows + 15) / 16);
+  const size_t sums = (size_t)slots * (tensor ? kCapG : ma * mb);
   void* more = nullptr;
-  IWF_TRY(contract_batch(engine, sc, &bt, sizeof(double2) * kCapG * ((size_t)slots + 1), &more));
+  IWF_TRY(contract_batch(engine, sc, &bt, sizeof(double2) * (kCapG + sums), &more));
   double2 *out = static_cast<double2*>(more), *part = out + kCapG;
   BlockList LA{}, LB{};
   LA.p[0] = A; LA.nb = 1; LA.b = ma;
   LB.p[0] = B; LB.nb = 1; LB.b = mb;
   IWF_TRY(gram<double>(bt, LA, LB, nrows, out, part, slots, st, false));
   IWF_CUDA(cudaMemcpyAsync(G, out, sizeof(double2) * (size_t)ma * mb, cudaMemcpyDeviceToDevice, st));
-  return contract_finish(bt, st);
+  return contract_finish(bt, sc);
 }
 
 iwf_status iwf_block_update(int engine, long long nrows, const void* S, int m, const void* C,
@@ -535,7 +582,7 @@ iwf_status iwf_block_update(int engine, long long nrows, const void* S, int m, c
   LS.p[0] = S; LS.nb = 1; LS.b = m;
   IWF_TRY(block_update<double>(bt, LS, nrows, static_cast<const double2*>(C), nullptr, m * q, q,
                                Y, nullptr, subtract != 0, st));
-  return contract_finish(bt, st);
+  return contract_finish(bt, sc);
 }
 
 }  // extern "C"
