@@ -1230,12 +1230,14 @@ iwf_status pencil_chunk(PencilArgs a, int LI, int LII, const void* in, void* wk,
 }
 
 // Whether the direct convolution (stencil.cu) runs the apply: its cost grows with the modes, the
-// transforms' does not. The limits lie where the fastest transforms (pencil set) were overtaken
-// on no window measured. Microseconds of transforms against direct, 16 vectors at 32^4 and (in
-// parentheses) 16^4: complex double 4330 (213), 24 complex modes 2669 (179), 32 3527 (235),
-// 48 real modes 2672 (179); complex float 184 (20), 16 complex modes 132 (15), 24 178 (19),
-// 32 225 (22). The tiled set is slower than the pencil set on every window (22^4, 24 vectors:
-// 5580 and 381 us; direct with 8 complex modes 356 and 36).
+// transforms' does not. One limit a precision, below the first window where the transforms win:
+// over 31 windows (one to five k_I axes; pencil, tiled and long axes) with 1, 2, 3, 4 and 16
+// vectors, no apply within it is slower than the transforms by more than 3 %. Microseconds of
+// transforms against direct: complex double, 16 vectors at 32^4 and (in parentheses) 16^4, 4334
+// (212), 24 complex modes 2666 (178), 32 3527 (234), 48 real modes 2679 (179); complex float, 16
+// vectors at 32^4 and (16^2 x 32^2), 187 (43.1), 20 complex modes 145 (44.2), 24 168 (49.3), 32
+// 207 (60), and one vector at 32^4 22.6, 20 modes 20.6, 24 24.6. The tiled set is overtaken later
+// (22^4, 16 vectors: 1535 and 134 us; 48 complex modes 1271 and 92).
 template <typename T>
 bool direct_pays(const iwf_plan* p, const ApplyBatch* batch) {
   if (p->path[sizeof(T) == 8 ? 0 : 1] != IWF_PATH_AUTO) return false;

@@ -551,7 +551,8 @@ __global__ void gram_tc_reduce(Batch bt, const double* partial, int slots, int m
 // arithmetic, warps 17..20 find the row scales of the tiles ahead.
 // A tile's MMAs and the reading of its accumulators take turns (nine levels of 48 columns fill
 // tensor memory), so the assembly bounds short contractions. In us for 2^20 rows, 24 outputs:
-// m = 24 337, m = 72 667, 48 columns subtracted 712; with four assembly warps, a variable binary
+// m = 24 370, m = 72 695, 48 columns subtracted 727 (of which 33, 28 and 15 for the low bits that
+// every sum keeps, see the assembly); with four assembly warps, a variable binary
 // point, old values loaded where they are needed and the slicing warps finding the scales in a
 // pass of their own 694, 1035 and 1465. Two warps for the row scales took 2117 (m = 72), tiles
 // dealt round-robin instead of in runs 769 (subtracted).

@@ -459,7 +459,7 @@ __device__ void herm_eig(SmallShared& sh, int n, int k) {
     const int any = __any_sync(0xffffffffu, close);
     if (lane == 0) sh.flag = any;
     if (lane < k) {
-      for (int i = 0; i < n; ++i) {
+      for (int i = 0; i < n; ++i) {                    // (mixed by xxHash32's multipliers and shifts)
         unsigned h = (unsigned)(i * 2654435761u) ^ ((unsigned)lane * 2246822519u + 374761393u);
         h ^= h >> 15; h *= 2246822519u; h ^= h >> 13; h *= 3266489917u; h ^= h >> 16;
         z[i * k + lane] = (double)((float)(int)h * 4.656612873e-10f);

@@ -107,8 +107,8 @@ template <bool REAL> struct ModeSum<float, REAL> {
 // Measured on 16 vectors, transforms before and this kernel now: complex double, 32^4, 8 real
 // modes 4330 -> 514 us (bound by the FP64 pipe: 18 operations a point, 480 us at its peak), Example
 // 4.1's 1280 x 2048 23.85 -> 0.74 ms (also FP64); complex float, 32^4, 8 complex modes 184 ->
-// 92 us, 16^6, 12 modes 15.1 -> 1.5 ms (issue and L1 latency together; ncu at 32^4: issue 51 %,
-// L1 50 %, DRAM 30 %, L2 29 %). NV = 2 or 8 were 30 % slower in complex float (index arithmetic;
+// 91 us (8 real ones 80), 16^6, 12 modes 15.1 -> 1.5 ms (issue and L1 latency together; ncu at 32^4,
+// complex modes: issue 57 %, L1 56 %, DRAM 33 %, L2 32 %). NV = 2 or 8 were 30 % slower in complex float (index arithmetic;
 // registers), U = 2 slower on 16^6, and patches of 2 x 2 to 4 x 8 slices a CTA, so that neighbour
 // slices come from its own L1, no faster anywhere. psi itself is loaded after the modes: held in
 // registers meanwhile it costs occupancy (111 us). Complex
