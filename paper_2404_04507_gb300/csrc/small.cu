@@ -10,8 +10,8 @@
 //     chains that do not depend on one another on different quarters of the SM;
 //   - bisection, which needs no last bit, counts eigenvalues in double-float arithmetic on the
 //     FP32 pipes (5x the FP64 rate); inverse iteration and Rayleigh quotients are FP64.
-// Measured on one GB300, Rayleigh-Ritz with 72 basis vectors and 24 pairs: 1.24 ms (reduction 0.50,
-// bisection 0.06, inverse iteration 0.11, back-transformation 0.24, P coefficients 0.33), m = 12
+// Measured on one GB300, Rayleigh-Ritz with 72 basis vectors and 24 pairs: 1.21 ms (reduction 0.50,
+// bisection 0.06, inverse iteration 0.11, back-transformation 0.24, P coefficients 0.30), m = 12
 // with 4 pairs 0.11 ms. Cyclic Jacobi in double-float arithmetic, which this replaced, took 6.2
 // and 0.30 ms (8 to 13 sweeps of 71 rounds at about 19k cycles) and left residuals near 1e-10 on
 // matrices with entries near 10^3; errors are now those of FP64 (residuals 2e-16 |A|).
@@ -778,20 +778,11 @@ __device__ void small_multiply(const double2* Y, const double2* T, double2* Z, i
   __syncthreads();
 }
 
-// Sum over the warp, in every lane.
-__device__ __forceinline__ double2 warp_sum(double2 s) {
-  for (int o = 16; o; o >>= 1) {
-    s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
-    s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
-  }
-  return s;
-}
-
 // First round of the P coefficients: Y = the columns in sh.B (m x b, rows below x_rows zero) minus
 // their projection on the orthonormal X in sh.A, scaled to unit norm and orthonormalised by
 // modified Gram-Schmidt; back to sh.B. Columns of norm up to 1e-12, and columns within 1e-7 of the
 // span of those before them, become zero with sh.keep 0. In FP64: double-float arithmetic took
-// 130 us less at 72 x 24, but left the span 1e-14 to 1e-13 off (now 4e-16).
+// 105 us less at 72 x 24, but left the span 1e-14 to 1e-13 off (now 4e-16).
 __device__ void p_columns_near(SmallShared& sh, int m, int b, int x_rows) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int kWarps = kSmallThreads / 32;
@@ -827,30 +818,41 @@ __device__ void p_columns_near(SmallShared& sh, int m, int b, int x_rows) {
     Y[c * ld + i] = s;
   }
   __syncthreads();
-  const auto dot = [&](const double2* a, const double2* y) {   // a^H y, in every lane
+  // eight lanes a column, four columns a warp: an FP64 instruction costs a warp the same with any
+  // number of lanes, and a sum over 32 lanes would take as many of them as the products
+  const int part = lane & 7, sub = lane >> 3;
+  const auto dots = [&](const double2* a, int j, bool live) {   // a^H y_j in the column's lanes
     double2 s = make_double2(0.0, 0.0);
-    for (int i = lane; i < m; i += 32) s = cmac_conj(a[i], y[i], s);
-    return warp_sum(s);
+    for (int i = part; live && i < m; i += 8) s = cmac_conj(a[i], Y[j * ld + i], s);
+    for (int o = 4; o; o >>= 1) {
+      s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+      s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+    }
+    return s;
   };
-  for (int c = warp; c < b; c += kWarps) {             // unit columns
-    const double n2 = dot(Y + c * ld, Y + c * ld).x;
+  for (int c0 = 4 * warp; c0 < b; c0 += 4 * kWarps) {  // unit columns
+    const int c = c0 + sub;
+    const bool live = c < b;
+    const double n2 = dots(Y + min(c, b - 1) * ld, c, live).x;
     const double f = n2 > 1e-24 ? rsqrt(n2) : 0.0;
-    for (int i = lane; i < m; i += 32) Y[c * ld + i] = make_double2(Y[c * ld + i].x * f, Y[c * ld + i].y * f);
+    for (int i = part; live && i < m; i += 8)
+      Y[c * ld + i] = make_double2(Y[c * ld + i].x * f, Y[c * ld + i].y * f);
   }
   __syncthreads();
   for (int l = 0; l < b; ++l) {
     const double2* yl = Y + l * ld;
-    for (int j = l + warp; j < b; j += kWarps) {
-      const double2 s = dot(yl, Y + j * ld);
-      if (lane == 0) G[j] = s;
+    for (int j0 = l + 4 * warp; j0 < b; j0 += 4 * kWarps) {
+      const int j = j0 + sub;
+      const double2 s = dots(yl, j, j < b);
+      if (part == 0 && j < b) G[j] = s;
     }
     __syncthreads();
     const double n2 = G[l].x;
     const bool on = n2 > 1e-14;
     const double f = on ? rsqrt(n2) : 0.0, f2 = f * f;
-    for (int j = l + 1 + warp; on && j < b; j += kWarps) {
+    for (int j = l + 1 + 4 * warp + sub; on && j < b; j += 4 * kWarps) {
       const double2 g = make_double2(-G[j].x * f2, -G[j].y * f2);
-      for (int i = lane; i < m; i += 32) Y[j * ld + i] = cmac(yl[i], g, Y[j * ld + i]);
+      for (int i = part; i < m; i += 8) Y[j * ld + i] = cmac(yl[i], g, Y[j * ld + i]);
     }
     __syncthreads();
     for (int i = tid; i < m; i += kSmallThreads) Y[l * ld + i] = make_double2(yl[i].x * f, yl[i].y * f);
